@@ -563,6 +563,7 @@ static int engine_setup(Engine &E, int nd, const pf_grid *g, const pf_params *p)
     CK(cudaMemset(E.d_flags, 0, sizeof(int) * 4));
     CK(cudaMalloc(&E.d_queue, sizeof(int) * 4));
     CK(cudaMalloc(&E.d_diag, sizeof(double) * (3 * diag_blocks() + 8)));
+    CK(cudaMemset(E.d_diag, 0, sizeof(double) * (3 * diag_blocks() + 8)));
     CK(cudaMalloc(&E.d_parts, sizeof(ParticleDev) * PF_MAX_PARTICLES));
     CK(cudaMalloc(&E.d_frep, sizeof(double) * 3 * PF_MAX_PARTICLES));
     return PF_OK;
@@ -1237,16 +1238,9 @@ static int engine_step(Engine &E, int64_t n, bool autotune)
     return PF_OK;
 }
 
-static int engine_sync(Engine &E)
+// the return code of the steps' flags (sticky when a bounded wait ran out)
+static int flags_rc(Engine &E, int flag)
 {
-    if (E.sticky) return E.sticky;
-    cudaError_t e = cudaStreamSynchronize(E.stream);
-    if (e != cudaSuccess) {
-        E.sticky = fail(PF_ECUDA, "asynchronous error: %s", cudaGetErrorString(e));
-        return E.sticky;
-    }
-    int flag = 0;
-    CK(cudaMemcpy(&flag, E.d_flags, sizeof(int), cudaMemcpyDeviceToHost));
     if (flag & 4) {
         E.sticky = fail(PF_ETIMEOUT, "a step kernel's bounded wait for its staged inputs ran out");
         return E.sticky;
@@ -1256,6 +1250,27 @@ static int engine_sync(Engine &E)
         return fail(PF_ENUMERIC, "a 16-bit order-parameter population reached the storage range and was "
                                  "saturated (raise the flow lattice's resolution or lower store_log2_scale[0])");
     return PF_OK;
+}
+
+// wait for the engine's stream
+static int engine_wait(Engine &E)
+{
+    cudaError_t e = cudaStreamSynchronize(E.stream);
+    if (e != cudaSuccess) {
+        E.sticky = fail(PF_ECUDA, "asynchronous error: %s", cudaGetErrorString(e));
+        return E.sticky;
+    }
+    return PF_OK;
+}
+
+static int engine_sync(Engine &E)
+{
+    if (E.sticky) return E.sticky;
+    int rc = engine_wait(E);
+    if (rc) return rc;
+    int flag = 0;
+    CK(cudaMemcpy(&flag, E.d_flags, sizeof(int), cudaMemcpyDeviceToHost));
+    return flags_rc(E, flag);
 }
 
 // tile tables and output buffer of the macroscopic pass, built once
@@ -1408,25 +1423,27 @@ static int engine_diag(Engine &E, int i, pf_diag *out)
     PfRange range("pf_diagnostics");
     if (!out) return fail(PF_EINVAL, "out is NULL");
     if (!E.inited[i]) return fail(PF_ESTATE, "pf_diagnostics before pf_init_fields");
-    int rc = engine_sync(E);
-    int nan_flag = 0;
-    if (rc == PF_ENUMERIC) CK(cudaMemcpy(&nan_flag, E.d_flags, sizeof(int), cudaMemcpyDeviceToHost));
-    if (rc && rc != PF_ENUMERIC) return rc;
-    rc = engine_macros(E, i);
+    if (E.sticky) return E.sticky;
+    // queued behind the steps, one wait: the results carry the steps' flags
+    int rc = engine_macros(E, i);
     if (rc) return rc;
     DomainDev dd = E.mem[i].d;
     dd.macro = E.d_macro;
-    double *partial = E.d_diag, *res = E.d_diag + 3 * diag_blocks();
-    launch_diag(dd, partial, res, E.wv, E.stream);
+    launch_diag(dd, E.d_diag, E.d_flags, E.wv, E.stream);
     CK(cudaGetLastError());
-    double h[3];
-    CK(cudaMemcpyAsync(h, res, sizeof(h), cudaMemcpyDeviceToHost, E.stream));
-    CK(cudaStreamSynchronize(E.stream));
+    double h[4];
+    const cudaError_t ce = cudaMemcpyAsync(h, E.d_diag + 3 * diag_blocks(), sizeof(h), cudaMemcpyDeviceToHost, E.stream);
+    rc = engine_wait(E);
+    if (rc) return rc;
+    CK(ce);
+    const int flag = (int)h[3];
+    rc = flags_rc(E, flag);
+    if (rc && rc != PF_ENUMERIC) return rc;
     out->mass = h[0];
     out->E_F = h[1];
     out->E_K = h[2];
     out->E_total = h[1] + h[2];
-    out->nan_flag = nan_flag;
+    out->nan_flag = flag;
     return PF_OK;
 }
 

@@ -43,7 +43,7 @@ bool launch_step3d_mixb(int tx, int ty, bool moving, int mode, int grid, cudaStr
 void launch_init(int prec, const DomainDev &Dm, int *flags, const double *phi0, const double *phi, const double *u,
                  const double *Pin, double *tmp, const ParticleDev *parts, int np, int wv, cudaStream_t s);
 int diag_blocks();
-void launch_diag(const DomainDev &Dm, double *partial, double *out, int wv, cudaStream_t s);
+void launch_diag(const DomainDev &Dm, double *scratch, const int *flags, int wv, cudaStream_t s);
 // near / far tile lists of a particle domain (single-cell / two-cells step)
 void launch_split_tiles(const StepArgs &a, int tx, int ty, unsigned char *sel, cudaStream_t s);
 // interface normal (dim planes of N) from Dm.macro's phi plane

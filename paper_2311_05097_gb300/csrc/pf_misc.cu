@@ -342,53 +342,144 @@ __global__ void k_init_f(DomainDev Dm, int *flags, const double *phi, const doub
 
 // ---- diagnostics --------------------------------------------------------------------------------
 
-// macro = [phi, rho, u (dim), P, mu, phi0] (double, x-fastest)
-__global__ void k_diag_partial(DomainDev Dm, double *partial, int wv)
+// Isotropic FD gradient (D2Q9 / D3Q19, classical weights, cs^2 = 1/3) of a dense
+// x-fastest double array at x of the rows of one neighbourhood: r[z][y] are
+// the rows z - 1 .. z + 1, y - 1 .. y + 1 (2D: r[1] only).  Opposite corners are
+// differenced once and shared by the components (24 FP64 operations in 3D, 10
+// in 2D: the FP64 pipe is what bounds the diagnostics).
+template <int DIM>
+__device__ __forceinline__ void diag_grad(const double *const (*r)[3], int xm, int x, int xp, double g[3])
+{
+    if constexpr (DIM == 2) {
+        const double a = r[1][2][xp] - r[1][0][xm], b = r[1][0][xp] - r[1][2][xm];
+        g[0] = (1.0 / 3.0) * (r[1][1][xp] - r[1][1][xm]) + (1.0 / 12.0) * (a + b);
+        g[1] = (1.0 / 3.0) * (r[1][2][x] - r[1][0][x]) + (1.0 / 12.0) * (a - b);
+        g[2] = 0.0;
+    } else {
+        const double a = r[1][2][xp] - r[1][0][xm], b = r[1][0][xp] - r[1][2][xm];  // (x, y) edges
+        const double c = r[2][1][xp] - r[0][1][xm], d = r[0][1][xp] - r[2][1][xm];  // (x, z) edges
+        const double e = r[2][2][x] - r[0][0][x], f = r[0][2][x] - r[2][0][x];      // (y, z) edges
+        g[0] = (1.0 / 6.0) * (r[1][1][xp] - r[1][1][xm]) + (1.0 / 12.0) * ((a + b) + (c + d));
+        g[1] = (1.0 / 6.0) * (r[1][2][x] - r[1][0][x]) + (1.0 / 12.0) * ((a - b) + (e + f));
+        g[2] = (1.0 / 6.0) * (r[2][1][x] - r[0][1][x]) + (1.0 / 12.0) * ((c - d) + (e - f));
+    }
+}
+
+// FP64 sums of phi, the free energy and the kinetic energy over macro = [phi,
+// rho, u (dim), P, mu, phi0] (double, x-fastest), and the flags of the steps.
+// Bound by the FP64 pipe (two thread instructions per clock and SM).  One warp
+// takes 32 cells of a row at a time (coalesced; the neighbours' rows are read
+// through L1), so no cell needs an integer division by nx ny; DIAG_BLOCKS x
+// 8 warps walk the row pieces with a fixed stride, and the last block to
+// finish adds the blocks' sums in order: the result depends on the grid's
+// sizes only.  grad phi0 (or W) is skipped by warps that see only zeros there.
+// Before (120 blocks, a contiguous run of cells per thread, a second launch for
+// the final sum, the steps' flags read apart): a pf_diagnostics call took 82 us
+// on 250 x 223 and 20.4 ms on 256^3; now 53 us and 4.5 ms, of which 1.85 ms
+// are the macroscopic pass.
+template <int DIM>
+__global__ void __launch_bounds__(256) k_diag(DomainDev Dm, double *partial, unsigned int *ticket, const int *flags,
+                                              double *out, int wv)
 {
     const DevParams &p = Dm.p;
-    const int dim = p.dim;
-    const long long N = (long long)Dm.nx * Dm.ny * Dm.nz;
+    const int nx = Dm.nx, ny = Dm.ny;
+    const long long N = (long long)nx * ny * Dm.nz;
     const double *phi = Dm.macro, *rho = Dm.macro + N, *u = Dm.macro + 2 * N;
-    const double *phi0 = Dm.macro + (2 + dim + 2) * N;
+    const double *phi0 = Dm.macro + (2 + DIM + 2) * N;
     const double *Wf = phi0 + N, *Vf = phi0 + 2 * N;  // own particle angles only
+    const double *wet = wv ? Wf : phi0;
+    const double s = p.sigma, D = p.D, ct = p.cos_t;
+    const double c_e = 3.0 * s / (4.0 * D), c_g = 3.0 * D * s / 16.0, c_p = 9.0 * s / (2.0 * D),
+                 c_w = 3.0 * s / D, c_gw = 3.0 * D * s / 8.0;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int pieces = (nx + 31) / 32, rows = ny * Dm.nz;
+    const long long items = (long long)rows * pieces, nw = (long long)gridDim.x * (blockDim.x >> 5);
     double acc[3] = {0.0, 0.0, 0.0};
-    // each thread walks a fixed contiguous range: deterministic order
-    const long long nthr = (long long)gridDim.x * blockDim.x;
-    const long long per = (N + nthr - 1) / nthr;
-    const long long gtid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    for (long long o = gtid * per; o < N && o < (gtid + 1) * per; ++o) {
-        const int x = (int)(o % Dm.nx), y = (int)((o / Dm.nx) % Dm.ny), z = (int)(o / ((long long)Dm.nx * Dm.ny));
-        double g[3], g0[3];
-        fd_grad_lap(Dm, phi, x, y, z, g, nullptr);
-        fd_grad_lap(Dm, wv ? Wf : phi0, x, y, z, g0, nullptr);
-        const double ph = phi[o], p0 = phi0[o];
-        double g2 = 0.0, g0g = 0.0, u2 = 0.0;
-        for (int a = 0; a < dim; ++a) {
-            g2 += g[a] * g[a];
-            g0g += g0[a] * g[a];
-            u2 += u[a * N + o] * u[a * N + o];
+    for (long long it = (long long)blockIdx.x * (blockDim.x >> 5) + warp; it < items; it += nw) {
+        const int row = (int)(it / pieces), x = (int)(it - (long long)row * pieces) * 32 + lane;
+        const int y = DIM == 2 ? row : row % ny, z = DIM == 2 ? 0 : row / ny;
+        const bool in = x < nx;
+        const int xc = in ? x : nx - 1, xm = xc == 0 ? nx - 1 : xc - 1, xp = xc == nx - 1 ? 0 : xc + 1;
+        const double *r[3][3], *q[3][3];
+#pragma unroll
+        for (int k = DIM == 2 ? 1 : 0; k < (DIM == 2 ? 2 : 3); ++k)
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                const int zz = DIM == 2 ? 0 : wrap1(z + k - 1, Dm.nz);
+                const long long o = ((long long)zz * ny + row_bc(Dm, y + j - 1)) * nx;
+                r[k][j] = phi + o;
+                q[k][j] = wet + o;
+            }
+        const long long o = (long long)row * nx + xc;
+        double g[3];
+        diag_grad<DIM>(r, xm, xc, xp, g);
+        // (the order of the loads and this test costs no FP64: bits are compared)
+        unsigned long long any = 0ull;
+#pragma unroll
+        for (int k = DIM == 2 ? 1 : 0; k < (DIM == 2 ? 2 : 3); ++k)
+#pragma unroll
+            for (int j = 0; j < 3; ++j)
+                any |= (unsigned long long)__double_as_longlong(q[k][j][xm]) |
+                       (unsigned long long)__double_as_longlong(q[k][j][xc]) |
+                       (unsigned long long)__double_as_longlong(q[k][j][xp]);
+        double g0g = 0.0;
+        if (__any_sync(0xffffffffu, any != 0ull)) {
+            double g0[3];
+            diag_grad<DIM>(q, xm, xc, xp, g0);
+#pragma unroll
+            for (int a = 0; a < DIM; ++a) g0g += g0[a] * g[a];
         }
-        const double s = p.sigma, D = p.D, ct = p.cos_t;
-        double e = 3.0 * s / (4.0 * D) * (1.0 - ph) * (1.0 - ph) * (1.0 + ph) * (1.0 + ph) +
-                   3.0 * D * s / 16.0 * g2 + 9.0 * s / (2.0 * D) * p0 * p0 * ph * ph;
+        if (!in) continue;  // (after the warp vote)
+        const double ph = phi[o], p0 = phi0[o];
+        double g2 = 0.0, u2 = 0.0;
+#pragma unroll
+        for (int a = 0; a < DIM; ++a) {
+            g2 += g[a] * g[a];
+            const double ua = u[a * N + o];
+            u2 += ua * ua;
+        }
+        double e = c_e * (1.0 - ph) * (1.0 - ph) * (1.0 + ph) * (1.0 + ph) + c_g * g2 + c_p * p0 * p0 * ph * ph;
         if (!wv)
-            e += 3.0 * s * ct / D * p0 * ph * (ph * ph + p0 * p0 - 1.0) + 3.0 * D * s * ct / 8.0 * g0g;
+            e += ct * (c_w * p0 * ph * (ph * ph + p0 * p0 - 1.0) + c_gw * g0g);
         else  // wetting energy summed per solid with its own angle (g0 = grad W)
-            e += 3.0 * s / D * (ph * (ph * ph - 1.0) * Wf[o] + ph * Vf[o]) + 3.0 * D * s / 8.0 * g0g;
+            e += c_w * (ph * (ph * ph - 1.0) * Wf[o] + ph * Vf[o]) + c_gw * g0g;
         acc[0] += ph;
         acc[1] += e;
         acc[2] += 0.5 * rho[o] * u2;
     }
-    __shared__ double red[256][3];
-    for (int c = 0; c < 3; ++c) red[threadIdx.x][c] = acc[c];
-    __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if ((int)threadIdx.x < s)
-            for (int c = 0; c < 3; ++c) red[threadIdx.x][c] += red[threadIdx.x + s][c];
+    __shared__ double red[8][3];
+    __shared__ bool last;
+    auto block_sum = [&](double *dst) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            double v = acc[c];
+#pragma unroll
+            for (int k = 16; k > 0; k >>= 1) v += __shfl_down_sync(0xffffffffu, v, k);
+            if (lane == 0) red[warp][c] = v;
+        }
         __syncthreads();
+        if (threadIdx.x < 3) {
+            double v = 0.0;
+            for (int w = 0; w < 8; ++w) v += red[w][threadIdx.x];
+            dst[threadIdx.x] = v;
+        }
+    };
+    block_sum(partial + 3 * blockIdx.x);
+    __threadfence();  // (the partial sums before the ticket)
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+        if (last) *ticket = 0u;  // for the next call on this stream
     }
-    if (threadIdx.x == 0)
-        for (int c = 0; c < 3; ++c) partial[blockIdx.x * 3 + c] = red[0][c];
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    acc[0] = acc[1] = acc[2] = 0.0;
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) acc[c] += __ldcg(partial + 3 * b + c);
+    block_sum(out);
+    if (threadIdx.x == 3) out[3] = (double)*flags;
 }
 
 // interface normal n = grad phi / |grad phi| from the macroscopic phi (central
@@ -442,23 +533,6 @@ void launch_split_tiles(const StepArgs &a, int tx, int ty, unsigned char *sel, c
 {
     k_split_tiles<<<(a.ntiles + 255) / 256, 256, 0, s>>>(a, tx, ty, sel);
     count_launches(1);
-}
-
-__global__ void k_diag_final(const double *partial, int nblocks, double *out)
-{
-    __shared__ double red[256][3];
-    double acc[3] = {0.0, 0.0, 0.0};
-    for (int b = threadIdx.x; b < nblocks; b += blockDim.x)
-        for (int c = 0; c < 3; ++c) acc[c] += partial[b * 3 + c];
-    for (int c = 0; c < 3; ++c) red[threadIdx.x][c] = acc[c];
-    __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if ((int)threadIdx.x < s)
-            for (int c = 0; c < 3; ++c) red[threadIdx.x][c] += red[threadIdx.x + s][c];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0)
-        for (int c = 0; c < 3; ++c) out[c] = red[0][c];
 }
 
 // ---- particles: repulsion (Sec. 4.5), per-tile partial sums, Newton-Euler (Eqs. 26, 28) --------
@@ -698,13 +772,22 @@ void launch_normal(const DomainDev &Dm, double *n, cudaStream_t s)
     count_launches(1);
 }
 
-int diag_blocks() { return 120; }
+// four blocks on each of the 152 SMs: the partial sums' table, and the order of
+// the sum, do not depend on the domain
+constexpr int DIAG_BLOCKS = 608;
+int diag_blocks() { return DIAG_BLOCKS; }
 
-void launch_diag(const DomainDev &Dm, double *partial, double *out, int wv, cudaStream_t s)
+// scratch: 3 diag_blocks() doubles of partial sums, 4 of results (sum phi, E_F,
+// E_K, flags), one zeroed ticket
+void launch_diag(const DomainDev &Dm, double *scratch, const int *flags, int wv, cudaStream_t s)
 {
-    k_diag_partial<<<diag_blocks(), 256, 0, s>>>(Dm, partial, wv);
-    k_diag_final<<<1, 256, 0, s>>>(partial, diag_blocks(), out);
-    count_launches(2);
+    double *out = scratch + 3 * DIAG_BLOCKS;
+    unsigned int *ticket = reinterpret_cast<unsigned int *>(out + 4);
+    if (Dm.p.dim == 2)
+        k_diag<2><<<DIAG_BLOCKS, 256, 0, s>>>(Dm, scratch, ticket, flags, out, wv);
+    else
+        k_diag<3><<<DIAG_BLOCKS, 256, 0, s>>>(Dm, scratch, ticket, flags, out, wv);
+    count_launches(1);
 }
 
 void launch_particle_update(ParticleDev *parts, int np, const double *partials, int ntiles,
