@@ -337,7 +337,8 @@ static int domain_alloc(DomainMem &m, int dim, const pf_grid *g, const DevParams
     const size_t rb = prec >= PF_PMIX_FP16 ? (size_t)d.plane * 8 : 0;
     const size_t ab = (size_t)naux * d.plane * aux_bytes(prec);
     const size_t pb = (size_t)d.plane * aux_bytes(prec);
-    const size_t total = 2 * fb + 2 * rb + 2 * ab + pb + 256 * 8 + 256 * 8;
+    const size_t tb = dim == 3 && prec != PF_P64 ? (size_t)d.plane * sizeof(float) : 0;  // phi of a 3D step
+    const size_t total = 2 * fb + 2 * rb + 2 * ab + pb + tb + 256 * 9 + 256 * 9;
     CK(cudaMalloc(&m.base, total));
     CK(cudaMemset(m.base, 0, total));
     char *c = (char *)m.base;
@@ -354,6 +355,7 @@ static int domain_alloc(DomainMem &m, int dim, const pf_grid *g, const DevParams
     d.aux[0] = take(ab);
     d.aux[1] = take(ab);
     d.phi0 = take(pb);
+    d.phi_t = tb ? (float *)take(tb) : nullptr;
     d.macro = nullptr;
     return PF_OK;
 }
@@ -428,9 +430,9 @@ static int domain_init(DomainMem &m, Staging &st, int dim, int prec, const doubl
 }
 
 // tile table of a set of domains (2D tiles of tx x ty; 3D column tiles of tx x ty
-// cells and zc planes)
+// cells and `chunks` chunks of at most zc planes)
 static void build_tiles(const std::vector<DomainMem *> &doms, int tx, int ty, std::vector<int> &tdom,
-                        std::vector<int2> &txy, int zc = ZCHUNK3D)
+                        std::vector<int2> &txy, int zc = ZCHUNK3D, int chunks = 1)
 {
     tdom.clear();
     txy.clear();
@@ -438,8 +440,8 @@ static void build_tiles(const std::vector<DomainMem *> &doms, int tx, int ty, st
         DomainDev &d = doms[k]->d;
         d.tiles_x = (d.nx + tx - 1) / tx;
         d.tiles_y = (d.ny + ty - 1) / ty;
-        d.zc = zc;
-        d.tiles_z = d.p.dim == 3 ? (d.nz + zc - 1) / zc : 1;
+        d.tiles_z = d.p.dim == 3 ? (d.nz + chunks * zc - 1) / (chunks * zc) : 1;
+        d.zc = (d.nz + chunks * d.tiles_z - 1) / (chunks * d.tiles_z);  // (even chunks)
         d.tile_base = (int)tdom.size();
         // 3D tiles encode (y tile, z chunk) as y + tiles_y * z
         for (int kz = 0; kz < d.tiles_z; ++kz)
@@ -622,6 +624,46 @@ static void drop_graph(Engine &E)
     }
 }
 
+// the 3D launches that run the two-cells-per-thread step (two chunks of z per tile)
+static bool pair3d(const Engine &E) { return E.dim == 3 && E.prec != PF_P64 && E.np == 0; }
+
+static int occupancy_any(const Engine &E, int tx, int ty, int mode);
+
+// Planes per z chunk of a 3D launch.  A tile costs its planes and a prologue
+// worth about three; n tiles resident on an SM take 0.55 + 0.45 n times as long as
+// one (latency-bound: measured 1.47 for two of the two-cells step), so short
+// chunks pay where the tiles would not fill the SMs and long ones where they do
+// many times over.  131 x 100 x 90 (FP32): 191 us per step at 32 planes a chunk,
+// 118 at 12; 256^3 (16-bit): 1109 us at 8, 1065 at 16, 1118 at 22.
+static int zchunk3d(const Engine &E, int tx, int ty)
+{
+    const int chunks = pair3d(E) ? 2 : 1, occ = std::max(1, occupancy_any(E, tx, ty, MODE_STEP));
+    const double full = 0.55 + 0.45 * occ;
+    int best = 1;
+    double tbest = 1e300;
+    for (int zc = 1; zc <= ZCHUNK3D; ++zc) {
+        long long tiles = 0, work = 0;
+        int planes = 1;
+        for (auto &m : E.mem) {
+            const int nz = m.d.nz, tz = (nz + chunks * zc - 1) / (chunks * zc);
+            const long long k = (long long)((m.d.nx + tx - 1) / tx) * ((m.d.ny + ty - 1) / ty) * tz;
+            const int pl = (nz + chunks * tz - 1) / (chunks * tz);
+            tiles += k;
+            work += k * (pl + 3);
+            planes = std::max(planes, pl);
+        }
+        // few tiles: those of the busiest SM; many: the whole work, and half a tile's tail
+        const long long n = (tiles + E.nsm - 1) / E.nsm, r = n % occ;
+        const double t = n > 2 * occ ? ((double)work / ((double)E.nsm * occ) + 0.5 * (planes + 3)) * full
+                                     : ((n / occ) * full + (r ? 0.55 + 0.45 * r : 0.0)) * (planes + 3);
+        if (t < tbest) {
+            tbest = t;
+            best = zc;
+        }
+    }
+    return best;
+}
+
 // upload the domain table and the tile table for shape (tx, ty)
 static int engine_tiles(Engine &E, int tx, int ty)
 {
@@ -629,7 +671,7 @@ static int engine_tiles(Engine &E, int tx, int ty)
     for (auto &m : E.mem) ds.push_back(&m);
     std::vector<int> tdom;
     std::vector<int2> txy;
-    build_tiles(ds, tx, ty, tdom, txy);
+    build_tiles(ds, tx, ty, tdom, txy, E.dim == 3 ? zchunk3d(E, tx, ty) : 1, pair3d(E) ? 2 : 1);
     if (E.d_tdom) cudaFree(E.d_tdom);
     if (E.d_txy) cudaFree(E.d_txy);
     E.d_tdom = nullptr;
@@ -758,6 +800,7 @@ static StepArgs step_args(const Engine &E, int par)
     a.items = E.d_items;
     a.nitems = E.nitems;
     a.strip_maps = E.d_maps;
+    a.dom1 = E.mem.size() == 1 ? &E.mem[0].d : nullptr;
     return a;
 }
 

@@ -198,10 +198,12 @@ struct DomainDev {
     void *rest[2];   // PMIX rest populations
     void *aux[2];    // lagged fields
     void *phi0;      // fixed indicator
+    float *phi_t;    // 3D, FP32 arithmetic: phi of the step under way (k_phi3d), else null
     double *macro;   // MODE_MACROS output: phi, rho, u(dim), P, mu, phi0 (double)
     int tile_base;   // index of this domain's first tile in the partial-sum table
     int tiles_x, tiles_y, tiles_z;
-    int zc;                // 3D: planes per z chunk of a tile (the last chunk may be shorter)
+    int zc;                // 3D: planes per z chunk of a tile (the last chunk may be shorter);
+                           // two chunks per tile in the two-cells-per-thread step
     DevParams p;
     KParams<float> kf;
     KParams<double> kd;
@@ -237,6 +239,7 @@ struct StepArgs {
     const int4 *items;              // strip kernel: work items (domain, x0, first row, end row)
     int nitems;
     const void *strip_maps;         // strip kernel: the tensor maps of every domain (128 bytes each)
+    const DomainDev *dom1;          // host copy of the only domain of the launch (3D two-cells step), or null
 };
 
 // ---- helpers -----------------------------------------------------------------------------------

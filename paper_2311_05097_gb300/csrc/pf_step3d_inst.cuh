@@ -2,7 +2,7 @@
 #pragma once
 
 #include "pf_internal.h"
-#include "pf_kernels3d.cuh"
+#include "pf_kernels3d_pair.cuh"
 
 namespace pf {
 
@@ -26,6 +26,29 @@ static bool run3d(int grid, cudaStream_t s, const StepArgs &a, int *occ)
     return true;
 }
 
+// the step of the FP32-arithmetic policies without particles: phi of every
+// cell, then the two-cells-per-thread update
+template <class P, int TX, int TY, bool EXT, bool UNIT, bool SINGLE>
+static bool run3d_pair(int grid, cudaStream_t s, const StepArgs &a, int *occ)
+{
+    auto kern = k_step3d_pair<P, TX, TY, EXT, UNIT, SINGLE>;
+    constexpr int smem = step3d_pair_smem<TX, TY>();
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return false;
+    if (occ) {
+        int n = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, TX * TY, smem) != cudaSuccess) n = 0;
+        *occ = n;
+        return true;
+    }
+    // eight pieces of a tile's planes: enough blocks of the light pass to fill
+    // the chip also where the tiles alone would not
+    const DomainDev d1 = SINGLE ? *a.dom1 : DomainDev{};
+    k_phi3d<P, TX, TY, EXT, SINGLE><<<dim3(a.ntiles, 8), TX * TY, 0, s>>>(a, d1);
+    kern<<<grid, TX * TY, smem, s>>>(a, d1);
+    count_launches(2);
+    return true;
+}
+
 template <class P, int TX, int TY, bool EXT>
 static bool dispatch3d_ext(bool moving, bool unit, int mode, int grid, cudaStream_t s, const StepArgs &a, int *occ)
 {
@@ -33,11 +56,17 @@ static bool dispatch3d_ext(bool moving, bool unit, int mode, int grid, cudaStrea
         return moving ? run3d<P, TX, TY, true, MODE_MACROS, EXT>(grid, s, a, occ)
                       : run3d<P, TX, TY, false, MODE_MACROS, EXT>(grid, s, a, occ);
     if constexpr (sizeof(typename P::real) == 4) {
-        // unit rates (FP32 arithmetic): the specialised collisions
-        if (unit && !moving) return run3d<P, TX, TY, false, MODE_STEP, EXT, true>(grid, s, a, occ);
+        if (!moving && a.dom1)
+            return unit ? run3d_pair<P, TX, TY, EXT, true, true>(grid, s, a, occ)
+                        : run3d_pair<P, TX, TY, EXT, false, true>(grid, s, a, occ);
+        if (!moving)
+            return unit ? run3d_pair<P, TX, TY, EXT, true, false>(grid, s, a, occ)
+                        : run3d_pair<P, TX, TY, EXT, false, false>(grid, s, a, occ);
+        return run3d<P, TX, TY, true, MODE_STEP, EXT>(grid, s, a, occ);
+    } else {
+        return moving ? run3d<P, TX, TY, true, MODE_STEP, EXT>(grid, s, a, occ)
+                      : run3d<P, TX, TY, false, MODE_STEP, EXT>(grid, s, a, occ);
     }
-    return moving ? run3d<P, TX, TY, true, MODE_STEP, EXT>(grid, s, a, occ)
-                  : run3d<P, TX, TY, false, MODE_STEP, EXT>(grid, s, a, occ);
 }
 
 // mode may carry MODE_EXT: a domain of the launch has walls

@@ -50,3 +50,46 @@ def test_diagnostics_row_pieces(pf, shape, walls):
         for k in ("mass", "E_F", "E_K"):
             assert abs(dg[k] - do[k]) <= 1e-12 * max(abs(do[k]), 1e-3), (k, dg[k], do[k])
         assert dg["nan_flag"] == 0
+
+
+@pytest.mark.parametrize("precision,tol", [("p32", dict(phi=5e-6, u=2e-4, P=2e-4)), ("fp16", dict(phi=1e-4, u=2e-2, P=2e-2))])
+@pytest.mark.parametrize("shape,walls,unit,model", [
+    ((4, 4, 4), False, True, 0), ((5, 9, 33), False, True, 0), ((5, 9, 33), True, True, 0), ((33, 8, 31), False, False, 0),
+    ((7, 17, 65), True, False, 0), ((67, 7, 32), False, True, 0), ((9, 10, 35), True, False, 1),
+])
+def test_pair_3d_chunk_edges(pf, precision, tol, shape, walls, unit, model):
+    """The 3D two-cells step: chunks of one plane and of unequal length, an empty
+    second chunk, tiles past the domain's end in x and y, walls on the tile's
+    first and last row, general rates and the Allen-Cahn lattice.  Bounds: ten
+    steps of a few FP32 roundings (6e-8) on fields of size 1 (phi), 0.01 (u) and
+    the flow populations' 2^-11 rounding in the 16-bit policy."""
+    if model and precision == "fp16":
+        pytest.skip("Allen-Cahn movers carry phi itself: the bound above is for Cahn-Hilliard ones")
+    c = W.small_case(shape, seed=11, solid=min(shape) > 6, theta_deg=75.0, u_amp=0.01, rho_ratio=2.0, mu_ratio=2.0)
+    c["params"].update(phase_model=model, solid_eps=0.1)
+    if not unit:
+        c["params"].update(s0=1.3, s1=0.9, s2=1.1, s3=1.2, s4=0.8, eta=0.0 if model else 0.3)
+    g, o = _pair(pf, c, 10, precision=precision, walls=walls)
+    gm, om = g.macros(), o.macros()
+    for k, t in tol.items():
+        assert np.abs(gm[k] - om[k]).max() <= t * max(np.abs(om[k]).max(), 1e-3), k
+    if precision == "fp16":
+        assert abs(g.diagnostics()["mass"] - c["phi"].sum()) <= 1e-12 * np.abs(c["phi"]).sum()
+
+
+def test_pair_3d_batch_equals_single_runs(pf):
+    """A batch of 3D domains (descriptors from the device table) and single runs
+    (descriptor as a kernel parameter) compute the same bits up to the packed
+    arithmetic's contraction: FP32 rounding over ten steps."""
+    cases = [W.small_case(s, seed=k, solid=True, theta_deg=60.0, u_amp=0.01, rho_ratio=2.0) for k, s in
+             enumerate([(9, 12, 33), (20, 8, 16), (13, 13, 13)])]
+    b = pf.Batch([c["shape"] for c in cases], [c["params"] for c in cases], precision="p32")
+    b.init_all([c["phi0"] for c in cases], [c["phi"] for c in cases], [c["u"] for c in cases])
+    b.step(10)
+    for i, c in enumerate(cases):
+        s = pf.Sim(c["shape"], precision="p32", **c["params"])
+        s.init(c["phi0"], c["phi"], c["u"])
+        s.step(10)
+        x, y = b.macros(i), s.macros()
+        for k in ("phi", "u"):
+            assert np.abs(x[k] - y[k]).max() <= 5e-6 * max(np.abs(y[k]).max(), 1e-3), k
