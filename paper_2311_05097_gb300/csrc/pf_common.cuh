@@ -197,8 +197,8 @@ struct DomainDev {
     void *f[2];      // population buffers
     void *rest[2];   // PMIX rest populations
     void *aux[2];    // lagged fields
-    void *phi0;      // fixed indicator
-    float *phi_t;    // 3D, FP32 arithmetic: phi of the step under way (k_phi3d), else null
+    void *phi0;      // fixed indicator (3D in FP32 arithmetic: then a plane for phi of the step
+                     // under way, k_phi3d)
     double *macro;   // MODE_MACROS output: phi, rho, u(dim), P, mu, phi0 (double)
     int tile_base;   // index of this domain's first tile in the partial-sum table
     int tiles_x, tiles_y, tiles_z;
@@ -208,6 +208,14 @@ struct DomainDev {
     KParams<float> kf;
     KParams<double> kd;
 };
+
+// Distance beyond R at which a particle's indicator 1/2 (1 + tanh(2 zeta / D)) is
+// exactly 0 in arithmetic type R: 10 D in FP64; 5 D in FP32, where 1 + tanhf(x)
+// is 0 for every x <= -10 (tanh(-10) is -1 within 5e-9, less than half the
+// spacing of FP32 there).  The smaller reach leaves fewer tiles and cells near
+// a particle, with the same results.
+template <class R>
+__device__ __forceinline__ double indicator_cut(const DevParams &p) { return sizeof(R) == 8 ? p.cut : 5.0 * p.D; }
 
 template <class R>
 __device__ __forceinline__ const KParams<R> &kparams(const DomainDev &d);

@@ -207,6 +207,7 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY>())) k_st
         const int x0 = txy.x * TX, y0 = txy.y * TY;
         const DevParams &p = Dm.p;
         const KParams<R> &kp = kparams<R>(Dm);
+        [[maybe_unused]] const double pcut = indicator_cut<R>(p);
 
         __syncthreads();  // previous tile's shared-memory readers are done
         if constexpr (MOVING) {
@@ -255,18 +256,18 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY>())) k_st
                 if (!EXT || !wall) dy = min_image(dy, ny);
                 const double ex = fmax(fabs(dx) - (0.5 * TX + 2.0), 0.0);
                 const double ey = fmax(fabs(dy) - (0.5 * TY + 2.0), 0.0);
-                const double lim = pp.R + p.cut + 1.0;
+                const double lim = pp.R + pcut + 1.0;
                 if (ex * ex + ey * ey < lim * lim) {
                     atomicOr(&s_near, 1ull << k);
                     s_pv[k][0] = (R)pp.R;
-                    s_pv[k][1] = (R)pp.R + (R)p.cut;
+                    s_pv[k][1] = (R)pp.R + (R)pcut;
                     s_pv[k][2] = (R)pp.u[0];
                     s_pv[k][3] = (R)pp.u[1];
                     s_pv[k][4] = (R)pp.w[2];
                     s_pv[k][5] = pp.own ? (R)pp.ct : R(0);
                     // a cell of the frames farther than nx/2 from this image is at
                     // least R + cut + 1 from every image when the box is this wide
-                    const double span = 2.0 * (pp.R + p.cut) + 8.0;
+                    const double span = 2.0 * (pp.R + pcut) + 8.0;
                     const bool fx = nx >= span + TX;
                     const bool fy = (EXT && wall) ? !wall_tile : ny >= span + TY;
                     if (fx && fy) {
@@ -288,7 +289,7 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY>())) k_st
             if ((fast >> k) & 1ull)
                 return particle_phi0_rel<R>(R(cx) - s_pcx[k], R(cy) - s_pcy[k], s_pv[k][0], s_pv[k][1], Dr,
                                             rx, ry);
-            return particle_phi0<R, EXT>(pp, gx, gy, nx, nyw, p.D, p.cut, rx, ry);
+            return particle_phi0<R, EXT>(pp, gx, gy, nx, nyw, p.D, pcut, rx, ry);
         };
 
         const ST *fs = reinterpret_cast<const ST *>(Dm.f[A.par]);

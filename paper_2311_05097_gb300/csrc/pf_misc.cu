@@ -521,7 +521,7 @@ __global__ void k_split_tiles(StepArgs A, int tx, int ty, unsigned char *sel)
         dy = min_image(dy, ny);
         const double ex = fmax(fabs(dx) - (0.5 * tx + 2.0), 0.0);
         const double ey = fmax(fabs(dy) - (0.5 * ty + 2.0), 0.0);
-        const double lim = pp.R + Dm.p.cut + 1.0;
+        const double lim = pp.R + indicator_cut<float>(Dm.p) + 1.0;  // (FP32 arithmetic only)
         near = ex * ex + ey * ey < lim * lim;
     }
     sel[t] = near ? 1 : 0;
