@@ -338,7 +338,7 @@ static int domain_alloc(DomainMem &m, int dim, const pf_grid *g, const DevParams
     const size_t ab = (size_t)naux * d.plane * aux_bytes(prec);
     const size_t pb = (size_t)d.plane * aux_bytes(prec);
     const size_t tb = dim == 3 && prec != PF_P64 ? (size_t)d.plane * sizeof(float) : 0;  // phi of a 3D step
-    const size_t total = 2 * fb + 2 * rb + 2 * ab + pb + tb + 256 * 9 + 256 * 9;
+    const size_t total = 2 * fb + 2 * rb + 2 * ab + pb + tb + 256 * 8 + 256 * 8;
     CK(cudaMalloc(&m.base, total));
     CK(cudaMemset(m.base, 0, total));
     char *c = (char *)m.base;
@@ -354,8 +354,7 @@ static int domain_alloc(DomainMem &m, int dim, const pf_grid *g, const DevParams
     d.rest[1] = rb ? take(rb) : nullptr;
     d.aux[0] = take(ab);
     d.aux[1] = take(ab);
-    d.phi0 = take(pb);
-    d.phi_t = tb ? (float *)take(tb) : nullptr;
+    d.phi0 = take(pb + tb);
     d.macro = nullptr;
     return PF_OK;
 }

@@ -2,7 +2,7 @@
 // (the 3D extension of Sec. 3; see the readings of the 3D lattices in the
 // oracle), pull streaming, Hermite-moment MRT collision.
 //
-// A CTA owns a TX x TY column of cells and marches through ZC planes in z.
+// A CTA owns a TX x TY column of cells and marches through a chunk of planes in z.
 // Shared-memory rings hold the planes the stencils need:
 //   phi, phi0       planes z-2 .. z+2 on the tile + 2 frame (ring of 5),
 //   mu_phi          planes z-1 .. z+1 on the tile + 1 frame (ring of 4),
@@ -266,23 +266,79 @@ __device__ __forceinline__ R lap19(const R *lo, const R *mid, const R *hi, int x
     return R(1) / R(3) * (faces - R(6) * c) + R(1) / R(6) * (edges - R(12) * c);
 }
 
-template <class R>
-__device__ __forceinline__ R particle_phi0_3d(const ParticleDev &pp, int gx, int gy, int gz, int nx,
-                                              int ny, int nz, double D, double cut, R &rx, R &ry,
-                                              R &rz)
+// Domain and tile coordinates of tile t.  SINGLE: a launch over one domain,
+// whose descriptor D1 is a kernel parameter: its sizes, pointers and constants
+// are then operands from the constant bank and everything derived from the
+// block index is uniform, which frees about forty registers of a thread.
+// (build_tiles orders the tiles x, y, z chunk.)
+template <bool SINGLE>
+__device__ __forceinline__ const DomainDev &tile_of(const StepArgs &A, const DomainDev &D1, int t, int &tx, int &ty, int &tz)
 {
-    double dx = (double)gx - pp.x[0], dy = (double)gy - pp.x[1], dz = (double)gz - pp.x[2];
-    dx = min_image(dx, nx);
-    if (ny > 0) dy = min_image(dy, ny);  // ny <= 0: walls in y, no minimum image
-    dz = min_image(dz, nz);
-    rx = (R)dx;
-    ry = (R)dy;
-    rz = (R)dz;
-    const double r2 = dx * dx + dy * dy + dz * dz;
-    const double lim = pp.R + cut;
-    if (r2 >= lim * lim) return R(0);
-    const R r = sqrt((R)r2);
-    return R(0.5) * (R(1) + tanh(R(2) * ((R)pp.R - r) / (R)D));
+    if constexpr (SINGLE) {
+        const int r = t / D1.tiles_x;
+        tx = t - r * D1.tiles_x;
+        tz = r / D1.tiles_y;
+        ty = r - tz * D1.tiles_y;
+        return D1;
+    } else {
+        const DomainDev &Dm = A.doms[A.tile_dom[t]];
+        const int2 txy = A.tile_xy[t];
+        tx = txy.x;
+        tz = txy.y / Dm.tiles_y;
+        ty = txy.y - tz * Dm.tiles_y;
+        return Dm;
+    }
+}
+
+// the plane of phi of the step under way (k_phi3d)
+__device__ __forceinline__ float *phi_of_step(const DomainDev &Dm) { return reinterpret_cast<float *>(Dm.phi0) + Dm.plane; }
+
+// One particle near a tile, in the arithmetic type: the image nearest to the
+// tile as whole cells (ix, iy, iz, in the tile's coordinates) and a fraction,
+// so that a cell's offset R(cell - i) - f is rounded once, as (R) of the FP64
+// difference is.
+template <class R>
+struct Near3 {
+    int ix, iy, iz, k, own, fast;  // fast 0: the box is too small for one image (or mirror rows), wrapped per cell
+    R fx, fy, fz, Rp, lim2, ct;
+    R u[3], w[3];
+};
+
+template <class R>
+__device__ __forceinline__ R near_phi0_3d(const Near3<R> &q, R rx, R ry, R rz, R D)
+{
+    const R r2 = rx * rx + ry * ry + rz * rz;
+    if (r2 >= q.lim2) return R(0);
+    return R(0.5) * (R(1) + tanh(R(2) * (q.Rp - sqrt(r2)) / D));
+}
+
+// Sums of six values over a warp by halving exchanges: each step a lane keeps
+// half of its components and adds its partner's (9 FP64 additions; six shuffle
+// trees take 30, and two FP64 lanes per SM and clock made them the force's
+// cost).  Lane 4 c holds the sum of component c.
+__device__ __forceinline__ double warp_sum6(const double v[6], int lane)
+{
+    double a[4], b[2];
+    const bool h16 = lane & 16, h8 = lane & 8, h4 = lane & 4;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const double up = i < 2 ? v[4 + i] : 0.0;
+        a[i] = (h16 ? up : v[i]) + __shfl_xor_sync(0xffffffffu, h16 ? v[i] : up, 16);
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) b[i] = (h8 ? a[2 + i] : a[i]) + __shfl_xor_sync(0xffffffffu, h8 ? a[i] : a[2 + i], 8);
+    double c = (h4 ? b[1] : b[0]) + __shfl_xor_sync(0xffffffffu, h4 ? b[0] : b[1], 4);
+    c += __shfl_xor_sync(0xffffffffu, c, 2);
+    return c + __shfl_xor_sync(0xffffffffu, c, 1);
+}
+
+// dynamic shared memory of the particle step: the near particles, each warp's
+// force and torque sums, and with own contact angles the W and V plane rings
+template <class R, int TX, int TY>
+constexpr size_t step3d_moving_smem(int np, bool wv)
+{
+    return (size_t)np * (sizeof(Near3<R>) + (TX * TY / 32) * 6 * sizeof(double)) +
+           (wv ? 2 * 5 * (size_t)(TX + 4) * (TY + 4) * sizeof(R) : 0);
 }
 
 // The step of FP64 and of free particles, and every policy's macroscopic pass
@@ -290,9 +346,22 @@ __device__ __forceinline__ R particle_phi0_3d(const ParticleDev &pp, int gx, int
 // EXT: the instantiation also handles domains with walls at the ends of y
 // UNIT: every domain of the launch has unit rates for its non-conserved
 // moments: the collisions above.
-template <class P, int TX, int TY, int ZC, bool MOVING, int MODE, bool EXT, bool UNIT = false>
-__global__ void __launch_bounds__(TX *TY, (sizeof(typename P::real) == 4 && !MOVING) ? 3 : 1) k_step3d(StepArgs A)
+// MOVING: a tile lists the particles whose indicator reaches its chunk (with
+// the image nearest to it), each plane visits those that reach the plane, a
+// warp's force terms are summed in FP64 and kept per warp until the chunk ends
+// (one barrier per chunk; before, every cell of every frame evaluated every
+// particle in FP64 and a barrier followed each particle and plane: 4055 thread
+// instructions per cell, one block of 202 registers per SM).  Three spheres in
+// 96 x 80 x 112 (FP32): 1240 us per step, 925 with the shorter chunks, 177 now;
+// with the FP64 minimum image per cell kept for boxes below 2 reach + tile, 501.  In FP32
+// arithmetic phi comes from k_phi3d's plane, as in k_step3d_pair, and the
+// domain's descriptor is a kernel parameter.
+template <class P, int TX, int TY, bool MOVING, int MODE, bool EXT, bool UNIT = false>
+__global__ void __launch_bounds__(TX *TY, (sizeof(typename P::real) == 4 && !MOVING) ? 3 : (MOVING && sizeof(typename P::real) == 4 ? 2 : 1))
+    k_step3d(const __grid_constant__ StepArgs A, const __grid_constant__ DomainDev D1)
 {
+    constexpr bool SINGLE = MOVING && MODE == MODE_STEP;             // (particles: single simulations only)
+    constexpr bool PHIT = SINGLE && sizeof(typename P::real) == 4;  // phi from k_phi3d
     using R = typename P::real;
     using ST = typename P::store;
     using AX = typename P::aux;
@@ -307,33 +376,34 @@ __global__ void __launch_bounds__(TX *TY, (sizeof(typename P::real) == 4 && !MOV
     __shared__ int s_gy[TY + 6];   // wrapped row offsets y * pitch
     __shared__ int s_gyi[TY + 6];  // wrapped rows
     __shared__ int s_out[EXT ? TY + 6 : 1];  // walls: the row lies beyond a wall (mirror image)
-    __shared__ double s_red[2][NT / 32][6];  // warps' sums, double-buffered over particles
-    // particles with their own contact angle (MOVING with A.wv): W and V of
-    // every staged phi0 plane (the same ring of 5), in dynamic shared memory
-    // (2 * 5 * FP values of R; the launch passes none otherwise)
+    __shared__ int s_nn;                     // near particles of the tile
+    // MOVING: the near particles, each warp's sums of force and torque, then with
+    // A.wv W and V of every staged phi0 plane (the same ring of 5)
     extern __shared__ __align__(16) unsigned char s_dyn3d[];
-    R *const s_W = reinterpret_cast<R *>(s_dyn3d);
+    constexpr int NW = NT / 32;
+    double *const s_facc = reinterpret_cast<double *>(s_dyn3d);  // [near particle][warp][6]
+    Near3<R> *const s_near = reinterpret_cast<Near3<R> *>(s_facc + (MOVING ? A.np * NW * 6 : 0));
+    R *const s_W = reinterpret_cast<R *>(s_near + (MOVING ? A.np : 0));
     R *const s_V = s_W + 5 * FP;
 
     const int tid = threadIdx.x;
     const int lx = tid % TX, ly = tid / TX;
 
     for (int t = blockIdx.x; t < A.ntiles; t += gridDim.x) {
-        const DomainDev &Dm = A.doms[A.tile_dom[t]];
-        const int2 txy = A.tile_xy[t];
+        int tx, ty, tz;
+        const DomainDev &Dm = tile_of<SINGLE>(A, D1, t, tx, ty, tz);
         const int nx = Dm.nx, ny = Dm.ny, nz = Dm.nz;
         const int plane = (int)Dm.plane;  // 26 * plane < 2^31 (checked at create)
         const int zstride = Dm.pitch * ny;
-        const int x0 = txy.x * TX;
-        const int y0 = (txy.y % Dm.tiles_y) * TY;
+        const int x0 = tx * TX;
+        const int y0 = ty * TY;
         const int zc = Dm.zc;
-        const int z0 = (txy.y / Dm.tiles_y) * zc;
+        const int z0 = tz * zc;
         const DevParams &p = Dm.p;
         const KParams<R> &kp = kparams<R>(Dm);
 
         __syncthreads();
         const int wall = EXT ? Dm.wall_y : 0;
-        const int nyw = wall ? 0 : ny;  // minimum image in y only without walls
         for (int k = tid; k < TX + 6; k += NT) s_gx[k] = wrap_idx(x0 - 3 + k, nx);
         for (int k = tid; k < TY + 6; k += NT) {
             if constexpr (EXT) {
@@ -358,6 +428,100 @@ __global__ void __launch_bounds__(TX *TY, (sizeof(typename P::real) == 4 && !MOV
             }
         }
         __syncthreads();
+        if constexpr (MOVING) {
+            // the particles whose reach meets the box of the tile's frames and
+            // planes (minimum image, conservative by a cell), in their order
+            if (tid < 32) {
+                int n = 0;
+                for (int k0 = 0; k0 < A.np; k0 += 32) {
+                    const int k = k0 + tid;
+                    bool hit = false;
+                    Near3<R> q;
+                    if (k < A.np) {
+                        const ParticleDev &pp = A.parts[k];
+                        const double mid[3] = {x0 + 0.5 * (TX - 1), y0 + 0.5 * (TY - 1), z0 + 0.5 * (zc - 1)};
+                        const double ext[3] = {0.5 * TX + 2.0, 0.5 * TY + 2.0, 0.5 * zc + 2.0};
+                        const int n3[3] = {nx, ny, nz}, len[3] = {TX, TY, zc};
+                        const double reach = pp.R + indicator_cut<R>(p);
+                        double c[3], e2 = 0.0;
+                        bool fast = true;
+#pragma unroll
+                        for (int a = 0; a < 3; ++a) {
+                            double dd = mid[a] - pp.x[a];
+                            const bool bounded = a == 1 && wall;
+                            if (!bounded) dd = min_image(dd, n3[a]);
+                            c[a] = mid[a] - dd;  // the image nearest to the tile
+                            const double ex = fmax(fabs(dd) - ext[a], 0.0);
+                            e2 += ex * ex;
+                            // with walls rows beyond them are mirror rows: their cells are not
+                            // where the table says
+                            fast = fast && (bounded ? !(y0 - 3 < 0 || y0 + TY + 3 > ny) : n3[a] >= 2.0 * reach + 6.0 + len[a]);
+                        }
+                        hit = e2 < (reach + 1.0) * (reach + 1.0);
+                        const double fl[3] = {floor(c[0]), floor(c[1]), floor(c[2])};
+                        q.ix = (int)fl[0] - x0;
+                        q.iy = (int)fl[1] - y0;
+                        q.iz = (int)fl[2] - z0;
+                        q.fx = (R)(c[0] - fl[0]);
+                        q.fy = (R)(c[1] - fl[1]);
+                        q.fz = (R)(c[2] - fl[2]);
+                        q.k = k;
+                        q.own = pp.own;
+                        q.fast = fast;
+                        q.Rp = (R)pp.R;
+                        q.lim2 = (R)reach * (R)reach;
+                        q.ct = pp.own ? (R)pp.ct : R(0);
+#pragma unroll
+                        for (int a = 0; a < 3; ++a) {
+                            q.u[a] = (R)pp.u[a];
+                            q.w[a] = (R)pp.w[a];
+                        }
+                    }
+                    const unsigned m = __ballot_sync(0xffffffffu, hit);
+                    if (hit) s_near[n + __popc(m & ((1u << tid) - 1u))] = q;
+                    n += __popc(m);
+                }
+                if (tid == 0) s_nn = n;
+            }
+            for (int q = tid; q < A.np * NW * 6; q += NT) s_facc[q] = 0.0;
+            __syncthreads();
+        }
+        [[maybe_unused]] const int nn = MOVING ? s_nn : 0;
+        // component of a cell's offset to a particle: its minimum image (min_image's
+        // rule, without FP64: the whole cells are wrapped before the one rounding)
+        [[maybe_unused]] auto wrapped = [](int d, R f, int n) -> R {
+            R r = R(d) - f;
+            const R half = R(0.5) * R(n);
+            if (r > half) r = R(d - n) - f;
+            else if (r < -half) r = R(d + n) - f;
+            return r;
+        };
+        // offset of cell (table cx, cy of the tile + 3 frame; plane z of the chunk's
+        // run z0 - 2 ..) to near particle q, and its indicator there
+        [[maybe_unused]] auto near_at = [&](const Near3<R> &q, int cx, int cy, int z, R &rx, R &ry, R &rz) -> R {
+            const int dx = cx - 3 - q.ix, dz = z - z0 - q.iz;
+            int dy = cy - 3 - q.iy;
+            if (q.fast) {
+                rx = R(dx) - q.fx;
+                ry = R(dy) - q.fy;
+                rz = R(dz) - q.fz;
+            } else {
+                rx = wrapped(dx, q.fx, nx);
+                rz = wrapped(dz, q.fz, nz);
+                if (EXT && wall) {
+                    dy = s_gyi[cy] - y0 - q.iy;  // (mirror rows; no image across a wall)
+                    ry = R(dy) - q.fy;
+                } else {
+                    ry = wrapped(dy, q.fy, ny);
+                }
+            }
+            return near_phi0_3d<R>(q, rx, ry, rz, (R)p.D);
+        };
+        // whether near particle q may reach plane z (uniform)
+        [[maybe_unused]] auto meets = [&](const Near3<R> &q, int z) -> bool {
+            const R dz = wrapped(z - z0 - q.iz, q.fz, nz);
+            return dz * dz < q.lim2;
+        };
         // a tile whose frames reach beyond a wall
         const bool wall_tile = EXT && wall && (y0 - 3 < 0 || y0 + TY + 3 > ny);
         // sign of the y-odd products T_xy, T_yz at table row r under a wall mirror
@@ -398,7 +562,21 @@ __global__ void __launch_bounds__(TX *TY, (sizeof(typename P::real) == 4 && !MOV
         auto phi_at = [&](int hx, int hy, int z, R *keep, ST *keepq) -> R {
             const int cx = hx + 1, cy = hy + 1;
             R acc;
-            if constexpr (P::MIX) {
+            if constexpr (PHIT) {
+                acc = phi_of_step(Dm)[cidx(cx, cy, zoff(z))];
+                if constexpr (!UNIT) {
+                    if (keep) {
+                        // (the rest population does not enter the collision's moments
+                        // beyond phi: keep[0] is set by the caller)
+#pragma unroll
+                        for (int i = P::MIX ? 1 : 0; i < 7; ++i) {
+                            const ST qv = ldg(fs + pull(0, i, cx, cy, z));
+                            keep[i] = Conv<P>::ld(qv, isc1);
+                            if (keepq) keepq[i] = qv;
+                        }
+                    }
+                }
+            } else if constexpr (P::MIX) {
                 acc = float_of_fixed(rs[cidx(cx, cy, zoff(z))]);
                 if (keep) keep[0] = acc;
 #pragma unroll
@@ -427,17 +605,17 @@ __global__ void __launch_bounds__(TX *TY, (sizeof(typename P::real) == 4 && !MOV
             const int cx = hx + 1, cy = hy + 1;
             R v = (R)ldg(ph0 + cidx(cx, cy, zoff(z)));
             if constexpr (MOVING) {
-                const int gx = s_gx[cx], gy = s_gyi[cy], gz = wrap_near(z, nz);
                 R dflt = v, w = R(0), vv = R(0);
-                for (int k = 0; k < A.np; ++k) {
+                for (int j = 0; j < nn; ++j) {
+                    const Near3<R> &q = s_near[j];
+                    if (!meets(q, z)) continue;
                     R rx, ry, rz;
-                    const R pk = particle_phi0_3d<R>(A.parts[k], gx, gy, gz, nx, nyw, nz, p.D, p.cut, rx, ry, rz);
+                    const R pk = near_at(q, cx, cy, z, rx, ry, rz);
                     v += pk;
                     if (Wo) {
-                        if (A.parts[k].own) {
-                            const R ck = (R)A.parts[k].ct;
-                            w += ck * pk;
-                            vv += ck * pk * pk * pk;
+                        if (q.own) {
+                            w += q.ct * pk;
+                            vv += q.ct * pk * pk * pk;
                         } else {
                             dflt += pk;
                         }
@@ -523,7 +701,7 @@ __global__ void __launch_bounds__(TX *TY, (sizeof(typename P::real) == 4 && !MOV
             load_T_plane(z0);
         }
         __syncthreads();
-        if (wall_tile) {
+        if (!PHIT && wall_tile) {  // (k_phi3d's plane is read at the mirror rows themselves)
             for (int z = z0 - 2; z <= z0 + 1; ++z) mirror_phi_plane(z);
             __syncthreads();
         }
@@ -537,7 +715,7 @@ __global__ void __launch_bounds__(TX *TY, (sizeof(typename P::real) == 4 && !MOV
             load_phi_plane(z + 2);
             if constexpr (MODE == MODE_STEP) load_T_plane(z + 1);
             __syncthreads();
-            if (wall_tile) {
+            if (!PHIT && wall_tile) {
                 mirror_phi_plane(z + 2);
                 __syncthreads();
             }
@@ -557,6 +735,13 @@ __global__ void __launch_bounds__(TX *TY, (sizeof(typename P::real) == 4 && !MOV
             R f1[7];
             ST q1[7];
             const R phi = phi_at(hx, hy, z, f1, q1);
+            // PHIT, 16-bit: k_phi3d left the exact phi where the rest population was
+            [[maybe_unused]] int sold = 0;
+            if constexpr (P::MIX && !(PHIT && UNIT)) {
+#pragma unroll
+                for (int i = 1; i < 7; ++i) sold += fix24_stored<ST>(q1[i]);
+                if constexpr (PHIT) f1[0] = float_of_fixed(rs[id] - fix24_to_rest(sold, p.klog2[0]));
+            }
             const R phi0 = s_p0[wrap_idx(z, 5)][hy * FX + hx];
             R gpx, gpy, gpz, gmx, gmy, gmz;
             grad19<R, FX>(plo, pmid, phi_hi, hx, hy, gpx, gpy, gpz);
@@ -671,14 +856,40 @@ __global__ void __launch_bounds__(TX *TY, (sizeof(typename P::real) == 4 && !MOV
                     usz = (jz + R(0.5) * Fz) * irho;
             R fpx = -phi0 * usx, fpy = -phi0 * usy, fpz = -phi0 * usz;
             if constexpr (MOVING) {
-                for (int k = 0; k < A.np; ++k) {
-                    const ParticleDev &pp = A.parts[k];
+                // the solids' velocity in the penalty force, and the hydrodynamic
+                // force and torque on each particle (Eq. 27): F = -sum rho phi0_k
+                // (u_s - u*), T = -sum r x (...), summed per warp in FP64
+                for (int j = 0; j < nn; ++j) {
+                    const Near3<R> &q = s_near[j];
+                    if (!meets(q, z)) continue;
                     R rx, ry, rz;
-                    const R pk = particle_phi0_3d<R>(pp, gx, gy, z, nx, nyw, nz, p.D, p.cut, rx, ry, rz);
+                    const R pk = near_at(q, lx + 3, ly + 3, z, rx, ry, rz);
+                    R vx = R(0), vy = R(0), vz = R(0);
                     if (pk != R(0)) {
-                        fpx += pk * ((R)pp.u[0] + (R)pp.w[1] * rz - (R)pp.w[2] * ry);
-                        fpy += pk * ((R)pp.u[1] + (R)pp.w[2] * rx - (R)pp.w[0] * rz);
-                        fpz += pk * ((R)pp.u[2] + (R)pp.w[0] * ry - (R)pp.w[1] * rx);
+                        vx = q.u[0] + q.w[1] * rz - q.w[2] * ry;
+                        vy = q.u[1] + q.w[2] * rx - q.w[0] * rz;
+                        vz = q.u[2] + q.w[0] * ry - q.w[1] * rx;
+                        fpx += pk * vx;
+                        fpy += pk * vy;
+                        fpz += pk * vz;
+                    }
+                    if constexpr (MODE == MODE_STEP) {
+                        const bool hit = valid && pk != R(0);
+                        if (!__any_sync(0xffffffffu, hit)) continue;
+                        double c6[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+                        if (hit) {
+                            const double fx = (double)(rho * pk * (vx - usx)), fy = (double)(rho * pk * (vy - usy)),
+                                         fz = (double)(rho * pk * (vz - usz));
+                            c6[0] = -fx;
+                            c6[1] = -fy;
+                            c6[2] = -fz;
+                            c6[3] = -((double)ry * fz - (double)rz * fy);
+                            c6[4] = -((double)rz * fx - (double)rx * fz);
+                            c6[5] = -((double)rx * fy - (double)ry * fx);
+                        }
+                        const double sum = warp_sum6(c6, tid & 31);
+                        const int comp = (tid & 31) >> 2;
+                        if ((tid & 3) == 0 && comp < 6) s_facc[(j * NW + (tid >> 5)) * 6 + comp] += sum;
                     }
                 }
             }
@@ -716,13 +927,7 @@ __global__ void __launch_bounds__(TX *TY, (sizeof(typename P::real) == 4 && !MOV
                     const long long N = (long long)nx * ny * nz;
                     const long long o = ((long long)z * ny + gy) * nx + gx;
                     double phv = (double)phi;
-                    if constexpr (P::MIX) {
-                        int sold = 0;
-#pragma unroll
-                        for (int i = 1; i < 7; ++i) sold += fix24_stored<ST>(q1[i]);
-                        const long long acc = rs[id] + fix24_to_rest(sold, p.klog2[0]);
-                        phv = double_of_fixed(acc);
-                    }
+                    if constexpr (P::MIX) phv = double_of_fixed(rs[id] + fix24_to_rest(sold, p.klog2[0]));
                     Dm.macro[0 * N + o] = phv;
                     Dm.macro[1 * N + o] = (double)rho;
                     Dm.macro[2 * N + o] = (double)ux;
@@ -830,9 +1035,7 @@ __global__ void __launch_bounds__(TX *TY, (sizeof(typename P::real) == 4 && !MOV
                     if constexpr (P::MIX) {
                         const R sc1 = kp.scale[0];
                         const int k1 = p.klog2[0];
-                        int bad = 0, sold = 0, snew = 0;
-#pragma unroll
-                        for (int i = 1; i < 7; ++i) sold += fix24_stored<ST>(q1[i]);
+                        int bad = 0, snew = 0;
 #pragma unroll
                         for (int i = 1; i < 7; ++i) {
                             ST qv = Conv<P>::st(f1[i], sc1);
@@ -841,7 +1044,7 @@ __global__ void __launch_bounds__(TX *TY, (sizeof(typename P::real) == 4 && !MOV
                             st_stream(fd + i * plane + id, qv);
                         }
                         // exact: sum of the cell's order-parameter populations is unchanged
-                        st_stream(rd + id, rs[id] + fix24_to_rest(sold - snew, k1));
+                        st_stream(rd + id, rs[id] + fix24_to_rest(PHIT ? -snew : sold - snew, k1));
                         if (bad) atomicOr(A.flags, 2);
                     } else {
 #pragma unroll
@@ -859,53 +1062,18 @@ __global__ void __launch_bounds__(TX *TY, (sizeof(typename P::real) == 4 && !MOV
                     st_stream(ad + 6 * plane + id, (AX)phi);
                     if (!isfinite(phi) || !isfinite(ux) || !isfinite(uy) || !isfinite(uz)) atomicOr(A.flags, 1);
                 }
-                if constexpr (MOVING) {
-                    for (int k = 0; k < A.np; ++k) {
-                        const ParticleDev &pp = A.parts[k];
-                        double c6[6] = {0, 0, 0, 0, 0, 0};
-                        bool hit = false;
-                        if (valid) {
-                            R rx, ry, rz;
-                            const R pk = particle_phi0_3d<R>(pp, gx, gy, z, nx, nyw, nz, p.D, p.cut, rx, ry, rz);
-                            if (pk != R(0)) {
-                                hit = true;
-                                const R vx = (R)pp.u[0] + (R)pp.w[1] * rz - (R)pp.w[2] * ry;
-                                const R vy = (R)pp.u[1] + (R)pp.w[2] * rx - (R)pp.w[0] * rz;
-                                const R vz = (R)pp.u[2] + (R)pp.w[0] * ry - (R)pp.w[1] * rx;
-                                const double fx = (double)(rho * pk * (vx - usx)), fy = (double)(rho * pk * (vy - usy)),
-                                             fz = (double)(rho * pk * (vz - usz));
-                                c6[0] = -fx;
-                                c6[1] = -fy;
-                                c6[2] = -fz;
-                                c6[3] = -((double)ry * fz - (double)rz * fy);
-                                c6[4] = -((double)rz * fx - (double)rx * fz);
-                                c6[5] = -((double)rx * fy - (double)ry * fx);
-                            }
-                        }
-                        // warp shuffle tree (skipped by warps whose terms are all 0),
-                        // warps in order; one barrier per particle and plane (the
-                        // buffer written here is next written after another barrier)
-                        const bool wany = __any_sync(0xffffffffu, hit);
-                        double(*red)[6] = s_red[k & 1];
-#pragma unroll
-                        for (int c = 0; c < 6; ++c) {
-                            double v = c6[c];
-                            if (wany) {
-#pragma unroll
-                                for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-                            }
-                            if ((tid & 31) == 0) red[tid >> 5][c] = v;
-                        }
-                        __syncthreads();
-                        if (tid < 6) {
-                            // per tile and plane: partial sums accumulate over the z loop in order
-                            double acc = 0.0;
-                            for (int wq = 0; wq < NT / 32; ++wq) acc += red[wq][tid];
-                            double *dst = A.partials + ((long long)k * 6 + tid) * A.ntiles + t;
-                            *dst = (z == z0 ? 0.0 : *dst) + acc;
-                        }
-                    }
-                }
+            }
+        }
+        if constexpr (MOVING && MODE == MODE_STEP) {
+            // the warps' sums in order; particles out of the chunk's reach: zero partials
+            __syncthreads();
+            for (int q = tid; q < 6 * A.np; q += NT) A.partials[(long long)q * A.ntiles + t] = 0.0;
+            __syncthreads();
+            for (int q = tid; q < 6 * nn; q += NT) {
+                const int j = q / 6, c = q - 6 * j;
+                double acc = 0.0;
+                for (int w = 0; w < NW; ++w) acc += s_facc[(j * NW + w) * 6 + c];
+                A.partials[((long long)s_near[j].k * 6 + c) * A.ntiles + t] = acc;
             }
         }
     }

@@ -32,35 +32,12 @@
 
 namespace pf {
 
-// Domain and tile coordinates of tile t.  SINGLE: a launch over one domain,
-// whose descriptor D1 is a kernel parameter: its sizes, pointers and constants
-// are then operands from the constant bank and everything derived from the
-// block index is uniform, which frees about forty registers of a thread.
-// (build_tiles orders the tiles x, y, z chunk.)
-template <bool SINGLE>
-__device__ __forceinline__ const DomainDev &tile_of(const StepArgs &A, const DomainDev &D1, int t, int &tx, int &ty, int &tz)
-{
-    if constexpr (SINGLE) {
-        const int r = t / D1.tiles_x;
-        tx = t - r * D1.tiles_x;
-        tz = r / D1.tiles_y;
-        ty = r - tz * D1.tiles_y;
-        return D1;
-    } else {
-        const DomainDev &Dm = A.doms[A.tile_dom[t]];
-        const int2 txy = A.tile_xy[t];
-        tx = txy.x;
-        tz = txy.y / Dm.tiles_y;
-        ty = txy.y - tz * Dm.tiles_y;
-        return Dm;
-    }
-}
-
 // phi of every cell of the tiles' columns: TX x TY threads, gridDim.y pieces of
-// a tile's 2 zc planes.  A streaming pass: 20 bytes in and 12 out per cell
+// the planes of a tile's chunks.  A streaming pass: 20 bytes in and 12 out per cell
 // (16-bit storage), 28 in and 4 out (FP32).
 template <class P, int TX, int TY, bool EXT, bool SINGLE>
-__global__ void __launch_bounds__(TX *TY) k_phi3d(const __grid_constant__ StepArgs A, const __grid_constant__ DomainDev D1)
+__global__ void __launch_bounds__(TX *TY) k_phi3d(const __grid_constant__ StepArgs A, const __grid_constant__ DomainDev D1,
+                                                   int chunks)
 {
     using ST = typename P::store;
     for (int t = blockIdx.x; t < A.ntiles; t += gridDim.x) {
@@ -69,7 +46,7 @@ __global__ void __launch_bounds__(TX *TY) k_phi3d(const __grid_constant__ StepAr
         const int nx = Dm.nx, ny = Dm.ny, nz = Dm.nz;
         const int x = tx * TX + threadIdx.x % TX, y = ty * TY + threadIdx.x / TX;
         if (x >= nx || y >= ny) continue;
-        const int z0 = tz * 2 * Dm.zc, zn = min(2 * Dm.zc, nz - z0);
+        const int z0 = tz * chunks * Dm.zc, zn = min(chunks * Dm.zc, nz - z0);
         const int per = (zn + gridDim.y - 1) / gridDim.y;
         const int za = z0 + blockIdx.y * per, zb = min(za + per, z0 + zn);
         const int plane = (int)Dm.plane, zstride = Dm.pitch * ny;
@@ -83,7 +60,7 @@ __global__ void __launch_bounds__(TX *TY) k_phi3d(const __grid_constant__ StepAr
         const bool bs = wall && y == 0, bn = wall && y == ny - 1;
         const int ys = (bs ? 4 * plane + own : 3 * plane + (y == 0 ? ny - 1 : y - 1) * Dm.pitch + x);
         const int yn = (bn ? 3 * plane + own : 4 * plane + (y == ny - 1 ? 0 : y + 1) * Dm.pitch + x);
-        float *out = Dm.phi_t;
+        float *out = phi_of_step(Dm);
         // BATCH planes' loads in flight before the first sum
         constexpr int BATCH = 4;
         for (int z = za; z < zb; z += BATCH) {
@@ -301,7 +278,7 @@ __global__ void __launch_bounds__(TX *TY, 2) k_step3d_pair(const __grid_constant
         ST *fd = reinterpret_cast<ST *>(Dm.f[A.par ^ 1]);
         const float *as = reinterpret_cast<const float *>(Dm.aux[A.par]);
         float *ad = reinterpret_cast<float *>(Dm.aux[A.par ^ 1]);
-        const float *ph0 = reinterpret_cast<const float *>(Dm.phi0), *pht = Dm.phi_t;
+        const float *ph0 = reinterpret_cast<const float *>(Dm.phi0), *pht = phi_of_step(Dm);
         const long long *rs = reinterpret_cast<const long long *>(Dm.rest[A.par]);
         long long *rd = reinterpret_cast<long long *>(Dm.rest[A.par ^ 1]);
 

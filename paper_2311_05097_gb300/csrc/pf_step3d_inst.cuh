@@ -9,10 +9,9 @@ namespace pf {
 template <class P, int TX, int TY, bool MOVING, int MODE, bool EXT, bool UNIT = false>
 static bool run3d(int grid, cudaStream_t s, const StepArgs &a, int *occ)
 {
-    auto kern = k_step3d<P, TX, TY, ZCHUNK3D, MOVING, MODE, EXT, UNIT>;
-    // particles with their own contact angle: the W and V plane rings (5
-    // planes of the tile + 2 frame each) in dynamic shared memory
-    const int dyn = (MOVING && a.wv) ? (int)(2 * 5 * (TX + 4) * (TY + 4) * sizeof(typename P::real)) : 0;
+    using R = typename P::real;
+    auto kern = k_step3d<P, TX, TY, MOVING, MODE, EXT, UNIT>;
+    const int dyn = MOVING ? (int)step3d_moving_smem<R, TX, TY>(a.np, a.wv) : 0;
     if (dyn && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn) != cudaSuccess)
         return false;
     if (occ) {
@@ -21,7 +20,12 @@ static bool run3d(int grid, cudaStream_t s, const StepArgs &a, int *occ)
         *occ = n;
         return true;
     }
-    kern<<<grid, TX * TY, dyn, s>>>(a);
+    const DomainDev d1 = a.dom1 ? *a.dom1 : DomainDev{};
+    if constexpr (MOVING && MODE == MODE_STEP && sizeof(R) == 4) {
+        k_phi3d<P, TX, TY, EXT, true><<<dim3(a.ntiles, 8), TX * TY, 0, s>>>(a, d1, 1);
+        count_launches(1);
+    }
+    kern<<<grid, TX * TY, dyn, s>>>(a, d1);
     count_launches(1);
     return true;
 }
@@ -43,7 +47,7 @@ static bool run3d_pair(int grid, cudaStream_t s, const StepArgs &a, int *occ)
     // eight pieces of a tile's planes: enough blocks of the light pass to fill
     // the chip also where the tiles alone would not
     const DomainDev d1 = SINGLE ? *a.dom1 : DomainDev{};
-    k_phi3d<P, TX, TY, EXT, SINGLE><<<dim3(a.ntiles, 8), TX * TY, 0, s>>>(a, d1);
+    k_phi3d<P, TX, TY, EXT, SINGLE><<<dim3(a.ntiles, 8), TX * TY, 0, s>>>(a, d1, 2);
     kern<<<grid, TX * TY, smem, s>>>(a, d1);
     count_launches(2);
     return true;
@@ -62,11 +66,14 @@ static bool dispatch3d_ext(bool moving, bool unit, int mode, int grid, cudaStrea
         if (!moving)
             return unit ? run3d_pair<P, TX, TY, EXT, true, false>(grid, s, a, occ)
                         : run3d_pair<P, TX, TY, EXT, false, false>(grid, s, a, occ);
-        return run3d<P, TX, TY, true, MODE_STEP, EXT>(grid, s, a, occ);
-    } else {
-        return moving ? run3d<P, TX, TY, true, MODE_STEP, EXT>(grid, s, a, occ)
-                      : run3d<P, TX, TY, false, MODE_STEP, EXT>(grid, s, a, occ);
     }
+    if (moving)
+        return unit ? run3d<P, TX, TY, true, MODE_STEP, EXT, true>(grid, s, a, occ)
+                    : run3d<P, TX, TY, true, MODE_STEP, EXT>(grid, s, a, occ);
+    if constexpr (sizeof(typename P::real) == 8)
+        return unit ? run3d<P, TX, TY, false, MODE_STEP, EXT, true>(grid, s, a, occ)
+                    : run3d<P, TX, TY, false, MODE_STEP, EXT>(grid, s, a, occ);
+    return false;
 }
 
 // mode may carry MODE_EXT: a domain of the launch has walls

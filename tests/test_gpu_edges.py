@@ -93,3 +93,34 @@ def test_pair_3d_batch_equals_single_runs(pf):
         x, y = b.macros(i), s.macros()
         for k in ("phi", "u"):
             assert np.abs(x[k] - y[k]).max() <= 5e-6 * max(np.abs(y[k]).max(), 1e-3), k
+
+
+# boxes wide enough for one image per tile (reach R + 10 D in FP64, R + 5 D in FP32 arithmetic), and
+# too small for it; particles across periodic faces, beside walls, of their own angle
+@pytest.mark.parametrize("precision,shape,walls", [
+    ("p64", (130, 20, 134), False), ("p64", (12, 17, 37), True), ("p32", (92, 96, 100), False), ("p32", (30, 92, 95), True),
+    ("fp16", (92, 23, 96), False), ("p32", (11, 9, 33), False),
+])
+def test_moving_3d_near_lists(pf, precision, shape, walls):
+    """The 3D particle step's lists of near particles: FP64 at 1e-12; the FP32 and
+    16-bit policies within a few roundings of four steps (FP32 6e-8, 16-bit
+    movers 2^-11 of sizes below 0.02), forces relative to the largest one."""
+    nz, ny, nx = shape
+    c = W.small_case(shape, seed=4, solid=False, u_amp=0.005, rho_ratio=1.0, mu_ratio=1.0)
+    R = min(4.0, 0.2 * min(shape))
+    # (no cell exactly half a box from a centre: its minimum image is not unique)
+    parts = [dict(x=(0.4, 0.5 * ny + 0.31, 0.6 * nz + 0.07), u=(0.01, 0.002, -0.004), w=(0.001, 0.0, 0.002), R=R, rho_p=2.0),
+             dict(x=(0.55 * nx + 0.03, 0.3 * ny + 0.11, nz - 0.7), u=(0.0, 0.01, 0.0), R=0.8 * R, rho_p=1.5, theta_deg=60.0),
+             dict(x=(nx - 5.2, ny - (R + 1.5 if walls else 0.2), 0.25 * nz + 0.09), u=(0.0, 0.0, 0.01), R=R, rho_p=1.2)]
+    for q in parts:
+        c["phi"] = (1.0 - W.disc(shape, q["x"], q["R"], 4.0)) * c["phi"]
+    g, o = _pair(pf, c, 4, precision=precision, particles=parts, walls=walls)
+    gm, om = g.macros(), o.macros()
+    tol = dict(p64=(1e-12, 1e-12, 1e-12), p32=(2e-6, 1e-4, 1e-4), fp16=(1e-4, 2e-2, 2e-2))[precision]
+    for k, t in zip(("phi", "u", "P"), tol):
+        assert np.abs(gm[k] - om[k]).max() <= t * max(np.abs(om[k]).max(), 1e-3), k
+    F = max(np.abs(np.array(o.particle(k).F)).max() for k in range(3))
+    for k in range(3):
+        pg, po = g.particle(k), o.particle(k)
+        assert np.abs(np.array(pg["x"]) - np.array(po.x)).max() <= 1e-6 * max(shape), k
+        assert np.abs(np.array(pg["F"]) - np.array(po.F)).max() <= (1e-11 if precision == "p64" else 2e-3) * F, k
