@@ -331,6 +331,8 @@ static int domain_alloc(DomainMem &m, int dim, const pf_grid *g, const DevParams
     d.p = dp;
     d.kf = make_kparams<float>(dp);
     d.kd = make_kparams<double>(dp);
+    d.uf = make_kunit<float>(dp);
+    d.ud = make_kunit<double>(dp);
     const int Q = dim == 2 ? 18 : 26;
     const int naux = 2 * dim + 1;
     const size_t fb = (size_t)Q * d.plane * store_bytes(prec);
@@ -463,6 +465,7 @@ struct Engine {
     int2 *d_txy = nullptr;
     int ntiles = 0;
     int tx = 32, ty = 8, cps = 0, grid = 0;  // tile shape, CTAs per SM, grid size
+    bool half = false;                       // 2D FP64: the 32 x 8 tiles run as 16 x 8 blocks
     int variant = 0;                         // 2D: 0 one cell per thread, 1 two, 2 two + staging,
                                              // 3 particle domain split: near tiles 0, far tiles 1
     unsigned char *d_sel = nullptr;          // variant 3: per tile 1 near a particle, 0 far
@@ -663,6 +666,23 @@ static int zchunk3d(const Engine &E, int tx, int ty)
     return best;
 }
 
+// 2D FP64 tiles of 32 x 8 run as 16 x 8 blocks where that leaves the busiest SM
+// fewer cells: the FP64 pipe bounds the step, so its time is that of the SM with
+// the most cells (a block's wider frames cost 2% more operations per cell).
+// 128^2: 64 tiles on 152 SMs, or 128 half tiles.
+static bool half_tiles(const Engine &E, int tx, int ty)
+{
+    if (E.dim != 2 || E.prec != PF_P64 || tx != 32 || ty != 8) return false;
+    long long n32 = 0, n16 = 0;
+    for (auto &m : E.mem) {
+        const long long rows = (m.d.ny + 7) / 8;
+        n32 += rows * ((m.d.nx + 31) / 32);
+        n16 += rows * ((m.d.nx + 15) / 16);
+    }
+    const long long c32 = (n32 + E.nsm - 1) / E.nsm * 256, c16 = (n16 + E.nsm - 1) / E.nsm * 128;
+    return 1.02 * (double)c16 < (double)c32;
+}
+
 // upload the domain table and the tile table for shape (tx, ty)
 static int engine_tiles(Engine &E, int tx, int ty)
 {
@@ -670,7 +690,8 @@ static int engine_tiles(Engine &E, int tx, int ty)
     for (auto &m : E.mem) ds.push_back(&m);
     std::vector<int> tdom;
     std::vector<int2> txy;
-    build_tiles(ds, tx, ty, tdom, txy, E.dim == 3 ? zchunk3d(E, tx, ty) : 1, pair3d(E) ? 2 : 1);
+    E.half = half_tiles(E, tx, ty);
+    build_tiles(ds, E.half ? 16 : tx, ty, tdom, txy, E.dim == 3 ? zchunk3d(E, tx, ty) : 1, pair3d(E) ? 2 : 1);
     if (E.d_tdom) cudaFree(E.d_tdom);
     if (E.d_txy) cudaFree(E.d_txy);
     E.d_tdom = nullptr;
@@ -731,6 +752,7 @@ static bool launch_any(const Engine &E, int tx, int ty, int mode, int grid, cons
     if (E.dim == 3)
         return launch_step3d(E.prec, tx, ty, E.np > 0,
                              mode | (any_walls(E) ? MODE_EXT : 0) | (all_unit(E) ? MODE_UNIT : 0), grid, E.stream, a);
+    if (E.half && mode == MODE_STEP && tx == 32 && ty == 8) tx = 16;
     return launch_step2d(E.prec, tx, ty, E.np > 0, mode | mode_flags(E), grid, E.stream, a);
 }
 
@@ -779,6 +801,7 @@ static int occupancy_any(const Engine &E, int tx, int ty, int mode)
     if (E.dim == 3)
         return occupancy_step3d(E.prec, tx, ty, E.np > 0,
                                 mode | (any_walls(E) ? MODE_EXT : 0) | (all_unit(E) ? MODE_UNIT : 0));
+    if (E.half && mode == MODE_STEP && tx == 32 && ty == 8) tx = 16;
     return occupancy_step2d(E.prec, tx, ty, E.np > 0, mode | mode_flags(E));
 }
 

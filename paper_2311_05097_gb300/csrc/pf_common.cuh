@@ -189,6 +189,23 @@ inline KParams<R> make_kparams(const DevParams &d)
     return k;
 }
 
+// Constants of the unit-rate step of one cell per thread, formed on the host: an
+// FP64 operation per thread costs as much for a constant as for a field.
+template <class R>
+struct KUnit {
+    R cs2, two_cs2, c3;  // cs^2, 2 cs^2, 1 - 3 cs^2
+    R h1c, qc;           // (1 - cs^2)/2, cs^2/4
+    R c2eta;             // cs^2 eta
+    R r0, g0;            // 1 - s0, 1 - s0/2
+};
+
+template <class R>
+inline KUnit<R> make_kunit(const DevParams &d)
+{
+    return {(R)d.cs2, (R)(2.0 * d.cs2), (R)(1.0 - 3.0 * d.cs2), (R)(0.5 * (1.0 - d.cs2)), (R)(0.25 * d.cs2),
+            (R)(d.cs2 * d.eta), (R)(1.0 - d.s0), (R)(1.0 - 0.5 * d.s0)};
+}
+
 // One domain of a (possibly batched) launch.
 struct DomainDev {
     int nx, ny, nz, pitch;
@@ -207,6 +224,8 @@ struct DomainDev {
     DevParams p;
     KParams<float> kf;
     KParams<double> kd;
+    KUnit<float> uf;
+    KUnit<double> ud;
 };
 
 // Distance beyond R at which a particle's indicator 1/2 (1 + tanh(2 zeta / D)) is
@@ -223,6 +242,13 @@ template <>
 __device__ __forceinline__ const KParams<float> &kparams<float>(const DomainDev &d) { return d.kf; }
 template <>
 __device__ __forceinline__ const KParams<double> &kparams<double>(const DomainDev &d) { return d.kd; }
+
+template <class R>
+__device__ __forceinline__ const KUnit<R> &kunit(const DomainDev &d);
+template <>
+__device__ __forceinline__ const KUnit<float> &kunit<float>(const DomainDev &d) { return d.uf; }
+template <>
+__device__ __forceinline__ const KUnit<double> &kunit<double>(const DomainDev &d) { return d.ud; }
 
 // Arguments of the step / macro kernels (2D and 3D).
 struct StepArgs {

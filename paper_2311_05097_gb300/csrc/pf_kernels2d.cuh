@@ -79,6 +79,55 @@ __device__ __forceinline__ void collide9(R f[9], const R heq[9], const R hF[9], 
     f[0] = m0 - m3 - m4 + m8;
 }
 
+// Unit rates (every rate of a non-conserved moment but s_2a and s_2b is 1, and
+// s_1phi): h* = heq + hF/2 for those moments.  The order-parameter lattice
+// after collision follows from phi, phi u + hF/2 = (j1, j2) and eta mu alone:
+// in raw moments m3 = m4 = cs2 eta mu, m8 = cs4 eta mu, m6, m7 = cs2 (j1, j2),
+// m5 = 0, and f = M_0^-1 m.
+template <class R>
+__device__ __forceinline__ void collide9_unit_phi(R f[9], R phi, R j1, R j2, R cs2_eta_mu, const KUnit<R> &ku)
+{
+    const R a = ku.h1c * cs2_eta_mu, b1 = ku.h1c * j1, b2 = ku.h1c * j2;  // (1 - cs2)/2
+    const R q8 = ku.qc * cs2_eta_mu, c1 = ku.qc * j1, c2 = ku.qc * j2;    // cs2/4
+    const R s = c1 + c2, d = c1 - c2;
+    f[0] = phi - R(2) * cs2_eta_mu + ku.cs2 * cs2_eta_mu;
+    f[1] = a + b1;
+    f[3] = a - b1;
+    f[2] = a + b2;
+    f[4] = a - b2;
+    f[5] = q8 + s;
+    f[7] = q8 - s;
+    f[8] = q8 + d;
+    f[6] = q8 - d;
+}
+
+// Flow lattice at unit rates: of its moments 0 (rate s0), 3, 4 (s_2a) and 5
+// (s_2b) are relaxed; h holds h* of moments 0 .. 5 (6, 7 are zero) and m8 is
+// its raw moment 8.
+template <class R>
+__device__ __forceinline__ void from_unit_flow(R f[9], const R h[6], R Pr, const KUnit<R> &ku)
+{
+    const R ch0 = ku.cs2 * h[0];
+    const R m3 = h[3] + ch0, m4 = h[4] + ch0;
+    const R m8 = ku.cs2 * (h[3] + h[4] + (ch0 - Pr));  // h8 = -cs2 P
+    const R q8 = R(0.25) * m8, q5 = R(0.25) * h[5], c1 = ku.qc * h[1], c2 = ku.qc * h[2];
+    const R sp = q8 + q5, sm = q8 - q5, cp = c1 + c2, cm = c1 - c2;
+    f[5] = sp + cp;
+    f[7] = sp - cp;
+    f[8] = sm + cm;
+    f[6] = sm - cm;
+    const R a3 = R(0.5) * (m3 - m8), a4 = R(0.5) * (m4 - m8), b1 = ku.h1c * h[1], b2 = ku.h1c * h[2];
+    f[1] = a3 + b1;
+    f[3] = a3 - b1;
+    f[2] = a4 + b2;
+    f[4] = a4 - b2;
+    f[0] = (h[0] - m3) - (m4 - m8);
+}
+
+// finite, by the exponent bits (FP64 comparisons run on the slow FP64 pipe)
+__device__ __forceinline__ bool finite_bits(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
+__device__ __forceinline__ bool finite_bits(float v) { return (__float_as_int(v) & 0x7f800000) != 0x7f800000; }
+
 // Isotropic central stencils on a shared-memory array (Sec. 3.2, last
 // paragraph): D2Q9 weights 4/9, 1/9, 1/36 with cs^2 = 1/3.
 template <class R, int W>
@@ -90,6 +139,17 @@ __device__ __forceinline__ void grad9(const R (*a)[W], int x, int y, R &gx, R &g
     const R third = R(1) / R(3), twelfth = R(1) / R(12);
     gx = third * (e - w) + twelfth * ((ne + se) - (nw + sw));
     gy = third * (n - s) + twelfth * ((ne + nw) - (se + sw));
+}
+
+// the same gradient with the corners' diagonal differences shared (10
+// operations instead of 12)
+template <class R, int W>
+__device__ __forceinline__ void grad9_diag(const R (*a)[W], int x, int y, R &gx, R &gy)
+{
+    const R d1 = a[y + 1][x + 1] - a[y - 1][x - 1], d2 = a[y - 1][x + 1] - a[y + 1][x - 1];
+    const R third = R(1) / R(3), twelfth = R(1) / R(12);
+    gx = third * (a[y][x + 1] - a[y][x - 1]) + twelfth * (d1 + d2);
+    gy = third * (a[y + 1][x] - a[y - 1][x]) + twelfth * (d1 - d2);
 }
 
 // the same gradient of the cubes a^3
@@ -146,19 +206,26 @@ __device__ __forceinline__ R particle_phi0_rel(R dx, R dy, R Rp, R lim, R D, R &
 }
 
 // Resident CTAs per SM requested from the register allocator: FP64 keeps its
-// registers (no cap); the 32 x 8 FP32/16-bit kernels trade a few spills for a
+// registers (no cap) but for the unit-rate step (132, capped at 128: 16 warps
+// per SM keep the FP64 pipe busy across the barriers); the 32 x 8 FP32/16-bit kernels trade a few spills for a
 // fourth CTA, 64 x 4 keeps three, 32 x 16 (the near tiles of the split step)
 // two; the autotuner picks among the shapes.
-template <class P, int TX, int TY>
+template <class P, int TX, int TY, bool CAP64>
 constexpr int step2d_min_blocks()
 {
-    return P::id == 0 ? 1 : (TX * TY > 256 ? 2 : ((TX == 32 && TY == 8) ? 4 : 3));
+    return P::id == 0 ? (CAP64 ? 512 / (TX * TY) : 1) : (TX * TY > 256 ? 2 : ((TX == 32 && TY == 8) ? 4 : 3));
 }
 
 // EXT: the instantiation also handles domains with walls at the ends of y;
 // without it the wall code is compiled out (it costs registers)
-template <class P, int TX, int TY, bool MOVING, int MODE, bool EXT>
-__global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY>())) k_step2d(StepArgs A)
+// UNIT: every domain of the launch has unit rates (DevParams::unit).  The order
+// parameter's populations are then only summed, the collisions take the short
+// forms above, and the four divisions of a cell become two.  In FP64 this is
+// what bounds the step: an SM retires two FP64 operations per cycle, and a cell
+// took about 540 of them (36 us per step of 128^2, 330 us for a batch of 0.27 M
+// cells).
+template <class P, int TX, int TY, bool MOVING, int MODE, bool EXT, bool UNIT = false>
+__global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY, UNIT && !MOVING && MODE == MODE_STEP>())) k_step2d(StepArgs A)
 {
     using R = typename P::real;
     using ST = typename P::store;
@@ -321,10 +388,8 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY>())) k_st
             if constexpr (P::MIX) {
                 const long long rv = rs[s_gy[cy] + s_gx[cx]];
                 acc = float_of_fixed(rv);
-                if (keep) {
-                    keep[0] = acc;
-                    rest_own = rv;
-                }
+                if (keep) keep[0] = acc;
+                if (keepq) rest_own = rv;
                 R movers = R(0);  // sum in stored units, scaled once
 #pragma unroll
                 for (int i = 1; i < 9; ++i) {
@@ -388,7 +453,7 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY>())) k_st
         }
         R f1[9];
         ST q1[9];
-        const R phi_own = phi_at(lx + 2, ly + 2, f1, q1);
+        const R phi_own = phi_at(lx + 2, ly + 2, UNIT ? nullptr : f1, q1);
         // PMIX: the cell's exact fixed-point phi; the pulled movers are dead after this
         [[maybe_unused]] long long racc = 0;
         if constexpr (P::MIX) {
@@ -398,7 +463,9 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY>())) k_st
             racc = rest_own + fix24_to_rest(sold, p.klog2[0]);
         }
         s_phi[ly + 2][lx + 2] = phi_own;
-        s_p0[ly + 2][lx + 2] = phi0_at(lx + 2, ly + 2);
+        const R p0_own = phi0_at(lx + 2, ly + 2);
+        s_p0[ly + 2][lx + 2] = p0_own;
+        [[maybe_unused]] int any_solid = p0_own != R(0);
         constexpr int RING = 4 * (TX + 4) + 4 * TY;
         for (int r = tid; r < RING; r += NT) {
             int hx, hy;
@@ -416,7 +483,9 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY>())) k_st
                 hx = c < 2 ? c : TX + c;
             }
             s_phi[hy][hx] = phi_at(hx, hy, nullptr, nullptr);
-            s_p0[hy][hx] = phi0_at(hx, hy);
+            const R p0 = phi0_at(hx, hy);
+            s_p0[hy][hx] = p0;
+            any_solid |= p0 != R(0);
         }
         if constexpr (MODE == MODE_STEP) {
             // w of the own cell from the lagged fields already in registers; the
@@ -454,7 +523,13 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY>())) k_st
                 }
             }
         }
-        __syncthreads();
+        // FP64: a frame without a solid skips the solid's terms of mu_phi, all
+        // zero (a third of stage B's operations)
+        bool solid_tile = true;
+        if constexpr (UNIT && sizeof(R) == 8)
+            solid_tile = __syncthreads_or(any_solid) || (MOVING && A.wv);
+        else
+            __syncthreads();
 
         // ---------------- stage B: mu_phi on tile+1 (Eq. 9) ----------------
         const R c_dw = kp.c_dw, c_lap = kp.c_lap, c_pen = kp.c_pen, c_wet = kp.c_wet,
@@ -462,8 +537,15 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY>())) k_st
         for (int r = tid; r < WX * WY; r += NT) {
             const int wx = r % WX, wy = r / WX;
             const int hx = wx + 1, hy = wy + 1;
-            const R ph = s_phi[hy][hx], p0 = s_p0[hy][hx];
+            const R ph = s_phi[hy][hx];
             const R lp = lap9<R, FX>(s_phi, hx, hy);
+            if constexpr (UNIT && sizeof(R) == 8) {
+                if (!solid_tile) {
+                    s_mu[wy][wx] = c_dw * ph * (ph - R(1)) * (ph + R(1)) - c_lap * lp;
+                    continue;
+                }
+            }
+            const R p0 = s_p0[hy][hx];
             const R base = c_dw * ph * (ph - R(1)) * (ph + R(1)) - c_lap * lp + c_pen * p0 * p0 * ph;
             bool own_wet = false;
             if constexpr (MOVING) {
@@ -486,17 +568,26 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY>())) k_st
         const int gx = x0 + lx, gy = y0 + ly;
         const bool valid = gx < nx && gy < ny;
         const int hx = lx + 2, hy = ly + 2, wx = lx + 1, wy = ly + 1;
+        // warps wholly beyond the domain have nothing to update
+        if constexpr (UNIT && !MOVING) {
+            if (!__any_sync(0xffffffffu, valid)) continue;
+        }
 
         const R phi = phi_own, phi0 = s_p0[hy][hx];
         R gpx, gpy, gmx, gmy;
-        grad9<R, FX>(s_phi, hx, hy, gpx, gpy);
-        grad9<R, WX>(s_mu, wx, wy, gmx, gmy);
+        if constexpr (UNIT) {
+            grad9_diag<R, FX>(s_phi, hx, hy, gpx, gpy);
+            grad9_diag<R, WX>(s_mu, wx, wy, gmx, gmy);
+        } else {
+            grad9<R, FX>(s_phi, hx, hy, gpx, gpy);
+            grad9<R, WX>(s_mu, wx, wy, gmx, gmy);
+        }
         const R mu = s_mu[wy][wx];
         const R drho = kp.drho;
         const R rho = drho * phi + kp.rhom;
         const R muv = kp.dmu * phi + kp.mum;
         // conservative Allen-Cahn option: theta n = (2/D)(1 - phi^2) grad phi/|grad phi|
-        const bool cac = EXT && p.phase_model == 1;
+        const bool cac = EXT && !UNIT && p.phase_model == 1;
         R tnx = R(0), tny = R(0);
         if (cac) {
             const R g2 = gpx * gpx + gpy * gpy;
@@ -513,7 +604,10 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY>())) k_st
         if constexpr (MODE == MODE_STEP) {
             // F_c = div(S u - u S)/2 from the previous step: (-d_y w, d_x w)/2
             R wgx, wgy;
-            grad9<R, WX>(s_w, wx, wy, wgx, wgy);
+            if constexpr (UNIT)
+                grad9_diag<R, WX>(s_w, wx, wy, wgx, wgy);
+            else
+                grad9<R, WX>(s_w, wx, wy, wgx, wgy);
             Fx += R(-0.5) * wgy;
             Fy += R(0.5) * wgx;
         } else {
@@ -587,10 +681,32 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY>())) k_st
 #pragma unroll
         for (int i = 0; i < 9; ++i) f2[i] = Conv<P>::ld(f2raw[i], isc2);
 
-        // u* (Eq. 36a)
-        const R jx = f2[1] - f2[3] + f2[5] - f2[6] - f2[7] + f2[8];
-        const R jy = f2[2] - f2[4] + f2[5] + f2[6] - f2[7] - f2[8];
-        const R irho = R(1) / rho;
+        // u* (Eq. 36a), the sums of the populations, and nu of Eq. 35 (1 - phi0
+        // bounded below by solid_eps)
+        R solid = R(1) - phi0;
+        const R seps = kp.solid_eps;
+        solid = solid < seps ? seps : solid;
+        R jx, jy, sum_f, irho, nu;
+        [[maybe_unused]] R m3r, m4r, m5r;  // raw moments 3, 4, 5
+        if constexpr (UNIT) {
+            const R a57 = f2[5] + f2[7], a68 = f2[6] + f2[8], d57 = f2[5] - f2[7], d68 = f2[6] - f2[8];
+            const R e24 = f2[2] + f2[4], m8r = a57 + a68;
+            m5r = a57 - a68;
+            m3r = (f2[1] + f2[3]) + m8r;
+            m4r = e24 + m8r;
+            sum_f = m3r + e24;
+            jx = (f2[1] - f2[3]) + (d57 - d68);
+            jy = (f2[2] - f2[4]) + (d57 + d68);
+            const R inv = R(1) / (rho * solid);  // one division for 1/rho and nu
+            irho = solid * inv;
+            nu = muv * inv;
+        } else {
+            jx = f2[1] - f2[3] + f2[5] - f2[6] - f2[7] + f2[8];
+            jy = f2[2] - f2[4] + f2[5] + f2[6] - f2[7] - f2[8];
+            sum_f = f2[1] + f2[2] + f2[3] + f2[4] + f2[5] + f2[6] + f2[7] + f2[8];
+            irho = R(1) / rho;
+            nu = muv / (rho * solid);
+        }
         const R usx = (jx + R(0.5) * Fx) * irho, usy = (jy + R(0.5) * Fy) * irho;
         // penalty force f = phi0 (u_s - u*) (Sec. 3.2, after Eq. 36)
         R fpx = -phi0 * usx, fpy = -phi0 * usy;
@@ -620,21 +736,26 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY>())) k_st
         const R Spx = (R)lag[2], Spy = (R)lag[3];
         const R php = (R)lag[4];
 
-        // relaxation rates (Eq. 35, 1 - phi0 bounded below by solid_eps)
-        R solid = R(1) - phi0;
-        const R seps = kp.solid_eps;
-        solid = solid < seps ? seps : solid;
-        const R nu = muv / (rho * solid);
+        // relaxation rates (Eq. 35)
         const R inv_s2a = R(0.5) + kp.two_over_1md0 * nu;
         const R inv_s2b = R(0.5) + kp.inv_cs2 * nu;
         const R Kf = kp.K;
         const R H = Kf * (kp.Hc0 - kp.Hc1 * inv_s2a);
         // pressure (Eq. 36b)
-        const R sum_f = f2[1] + f2[2] + f2[3] + f2[4] + f2[5] + f2[6] + f2[7] + f2[8];
-        const R ugr = ux * grx + uy * gry;
-        const R rus_u = (rho * ux - Sx) * ux + (rho * uy - Sy) * uy;
-        const R Su = Sx * ux + Sy * uy, Sup = Spx * upx + Spy * upy;
-        const R dt_term = R(2) * (ux * Ftx + uy * Fty) - (Su - Sup);
+        const R rux = rho * ux, ruy = rho * uy;
+        const R exx = (rux - Sx) * ux, eyy = (ruy - Sy) * uy, gxx = ux * grx, gyy = uy * gry;
+        const R dxx = Sx * ux - Spx * upx, dyy = Sy * uy - Spy * upy, wxx = ux * Ftx, wyy = uy * Fty;
+        R ugr, rus_u, dt_term;
+        if constexpr (UNIT) {
+            ugr = gxx + gyy;
+            rus_u = exx + eyy;
+            dt_term = R(2) * (wxx + wyy) - (dxx + dyy);
+        } else {
+            ugr = ux * grx + uy * gry;
+            rus_u = (rho * ux - Sx) * ux + (rho * uy - Sy) * uy;
+            const R Su = Sx * ux + Sy * uy, Sup = Spx * upx + Spy * upy;
+            dt_term = R(2) * (ux * Ftx + uy * Fty) - (Su - Sup);
+        }
         const R Pr = kp.Pfac * (sum_f + (R(0.5) + H) * ugr - kp.w0f * rus_u * kp.inv_1mcs2 +
                                  Kf * R(0.5) * dt_term);
 
@@ -660,64 +781,90 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY>())) k_st
             }
             continue;
         } else {
-            const R cs2 = kp.cs2, cs4 = kp.cs4;
-            // ---- order-parameter lattice (Eq. 30): Hermite equilibria and source
-            // (Allen-Cahn: eta mu -> phi, and cs^2 theta n joins the source)
-            const R eta_mu = cac ? phi : kp.eta * mu;
-            R heq[9], hF[9], S[9];
-            heq[0] = phi;
-            heq[1] = phi * ux;
-            heq[2] = phi * uy;
-            heq[3] = cs2 * (eta_mu - phi);
-            heq[4] = heq[3];
-            heq[5] = R(0);
-            heq[6] = R(0);
-            heq[7] = R(0);
-            heq[8] = cs4 * (phi - eta_mu);
-            hF[0] = R(0);
-            hF[1] = phi * ux - php * upx;  // d_t(phi u), explicit Euler
-            hF[2] = phi * uy - php * upy;
-            if (cac) {
-                hF[1] += cs2 * tnx;
-                hF[2] += cs2 * tny;
-            }
+            if constexpr (UNIT) {
+                const KUnit<R> &ku = kunit<R>(Dm);
+                // order parameter: phi u and half of d_t(phi u) (explicit Euler)
+                const R pux = phi * ux, puy = phi * uy;
+                collide9_unit_phi<R>(f1, phi, pux + R(0.5) * (pux - php * upx), puy + R(0.5) * (puy - php * upy),
+                                     ku.c2eta * mu, ku);
+                // flow (Eqs. 32-34): second-order equilibria and sources
+                const R inv_ab = R(1) / (inv_s2a * inv_s2b);  // one division for both rates
+                const R s2a = inv_s2b * inv_ab, s2b = inv_s2a * inv_ab;
+                const R m0 = f2[0] + sum_f, c3u = ku.c3 * ugr;
+                const R cross = Sx * uy + ux * Sy, crossp = Spx * upy + upx * Spy;
+                const R d3 = m3r - ku.cs2 * m0, d4 = m4r - ku.cs2 * m0;
+                const R q3 = R(2) * wxx + (ku.two_cs2 * gxx + (c3u - dxx));
+                const R q4 = R(2) * wyy + (ku.two_cs2 * gyy + (c3u - dyy));
+                const R q5 = (ux * Fty + Ftx * uy) + (ku.cs2 * (ux * gry + grx * uy) - R(0.5) * (cross - crossp));
+                R h[6];
+                h[0] = ku.r0 * m0 + ku.g0 * ugr;
+                h[1] = rux + R(0.5) * Ftx;
+                h[2] = ruy + R(0.5) * Fty;
+                // h - s (h - heq) + (1 - s/2) hF = (h + hF) + s (heq - h - hF/2)
+                h[3] = (d3 + q3) + s2a * ((Pr + exx) - (d3 + R(0.5) * q3));
+                h[4] = (d4 + q4) + s2a * ((Pr + eyy) - (d4 + R(0.5) * q4));
+                h[5] = (m5r + q5) + s2b * ((rux * uy - R(0.5) * cross) - (m5r + R(0.5) * q5));
+                from_unit_flow<R>(f2, h, Pr, ku);
+            } else {
+                const R cs2 = kp.cs2, cs4 = kp.cs4;
+                // ---- order-parameter lattice (Eq. 30): Hermite equilibria and source
+                // (Allen-Cahn: eta mu -> phi, and cs^2 theta n joins the source)
+                const R eta_mu = cac ? phi : kp.eta * mu;
+                R heq[9], hF[9], S[9];
+                heq[0] = phi;
+                heq[1] = phi * ux;
+                heq[2] = phi * uy;
+                heq[3] = cs2 * (eta_mu - phi);
+                heq[4] = heq[3];
+                heq[5] = R(0);
+                heq[6] = R(0);
+                heq[7] = R(0);
+                heq[8] = cs4 * (phi - eta_mu);
+                hF[0] = R(0);
+                hF[1] = phi * ux - php * upx;  // d_t(phi u), explicit Euler
+                hF[2] = phi * uy - php * upy;
+                if (cac) {
+                    hF[1] += cs2 * tnx;
+                    hF[2] += cs2 * tny;
+                }
 #pragma unroll
-            for (int k = 3; k < 9; ++k) hF[k] = R(0);
-            S[0] = kp.s0;
-            S[1] = S[2] = kp.s1phi;
-            S[3] = S[4] = S[5] = kp.s2;
-            S[6] = S[7] = kp.s3;
-            S[8] = kp.s4;
-            collide9<R>(f1, heq, hF, S, cs2);
+                for (int k = 3; k < 9; ++k) hF[k] = R(0);
+                S[0] = kp.s0;
+                S[1] = S[2] = kp.s1phi;
+                S[3] = S[4] = S[5] = kp.s2;
+                S[6] = S[7] = kp.s3;
+                S[8] = kp.s4;
+                collide9<R>(f1, heq, hF, S, cs2);
 
-            // ---- flow lattice (Eqs. 32-34)
-            heq[0] = R(0);
-            heq[1] = rho * ux;
-            heq[2] = rho * uy;
-            heq[3] = Pr + rho * ux * ux - Sx * ux;
-            heq[4] = Pr + rho * uy * uy - Sy * uy;
-            heq[5] = rho * ux * uy - R(0.5) * (Sx * uy + ux * Sy);
-            heq[6] = R(0);
-            heq[7] = R(0);
-            heq[8] = -cs2 * Pr;
-            const R c3 = R(1) - R(3) * cs2;
-            hF[0] = ugr;
-            hF[1] = Ftx;
-            hF[2] = Fty;
-            hF[3] = R(2) * ux * Ftx - (Sx * ux - Spx * upx) + R(2) * cs2 * ux * grx + c3 * ugr;
-            hF[4] = R(2) * uy * Fty - (Sy * uy - Spy * upy) + R(2) * cs2 * uy * gry + c3 * ugr;
-            hF[5] = ux * Fty + Ftx * uy - R(0.5) * ((Sx * uy + ux * Sy) - (Spx * upy + upx * Spy)) +
-                    cs2 * (ux * gry + grx * uy);
-            hF[6] = R(0);
-            hF[7] = R(0);
-            hF[8] = R(0);
-            S[0] = kp.s0;
-            S[1] = S[2] = kp.s1;
-            S[3] = S[4] = R(1) / inv_s2a;
-            S[5] = R(1) / inv_s2b;
-            S[6] = S[7] = kp.s3;
-            S[8] = kp.s4;
-            collide9<R>(f2, heq, hF, S, cs2);
+                // ---- flow lattice (Eqs. 32-34)
+                heq[0] = R(0);
+                heq[1] = rho * ux;
+                heq[2] = rho * uy;
+                heq[3] = Pr + rho * ux * ux - Sx * ux;
+                heq[4] = Pr + rho * uy * uy - Sy * uy;
+                heq[5] = rho * ux * uy - R(0.5) * (Sx * uy + ux * Sy);
+                heq[6] = R(0);
+                heq[7] = R(0);
+                heq[8] = -cs2 * Pr;
+                const R c3 = R(1) - R(3) * cs2;
+                hF[0] = ugr;
+                hF[1] = Ftx;
+                hF[2] = Fty;
+                hF[3] = R(2) * ux * Ftx - (Sx * ux - Spx * upx) + R(2) * cs2 * ux * grx + c3 * ugr;
+                hF[4] = R(2) * uy * Fty - (Sy * uy - Spy * upy) + R(2) * cs2 * uy * gry + c3 * ugr;
+                hF[5] = ux * Fty + Ftx * uy - R(0.5) * ((Sx * uy + ux * Sy) - (Spx * upy + upx * Spy)) +
+                        cs2 * (ux * gry + grx * uy);
+                hF[6] = R(0);
+                hF[7] = R(0);
+                hF[8] = R(0);
+                S[0] = kp.s0;
+                S[1] = S[2] = kp.s1;
+                S[3] = S[4] = R(1) / inv_s2a;
+                S[5] = R(1) / inv_s2b;
+                S[6] = S[7] = kp.s3;
+                S[8] = kp.s4;
+                collide9<R>(f2, heq, hF, S, cs2);
+            }
 
             if (valid) {
                 // populations (own cell; the next step pulls them)
@@ -751,7 +898,7 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY>())) k_st
                 ad[2 * plane + id] = (AX)Sx;
                 ad[3 * plane + id] = (AX)Sy;
                 ad[4 * plane + id] = (AX)phi;
-                if (!isfinite(phi) || !isfinite(ux) || !isfinite(uy)) atomicOr(A.flags, 1);
+                if (!finite_bits(phi) || !finite_bits(ux) || !finite_bits(uy)) atomicOr(A.flags, 1);
             }
 
             if constexpr (MOVING) {

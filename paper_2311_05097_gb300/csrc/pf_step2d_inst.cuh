@@ -10,10 +10,10 @@
 
 namespace pf {
 
-template <class P, int TX, int TY, bool MOVING, int MODE, bool EXT>
+template <class P, int TX, int TY, bool MOVING, int MODE, bool EXT, bool UNIT = false>
 static bool run2d(int grid, cudaStream_t s, const StepArgs &a, int *occ)
 {
-    auto kern = k_step2d<P, TX, TY, MOVING, MODE, EXT>;
+    auto kern = k_step2d<P, TX, TY, MOVING, MODE, EXT, UNIT>;
     if (occ) {
         int n = 0;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, TX * TY, 0) != cudaSuccess) n = 0;
@@ -149,8 +149,28 @@ static bool dispatch2d_strip(int tx, bool moving, bool cac, bool unit, bool wall
     }
 }
 
+template <class P, bool EXT, bool UNIT>
+static bool dispatch2d_step(int tx, int ty, bool moving, int grid, cudaStream_t s, const StepArgs &a, int *occ)
+{
+    if (tx == 32 && ty == 8)
+        return moving ? run2d<P, 32, 8, true, MODE_STEP, EXT, UNIT>(grid, s, a, occ)
+                      : run2d<P, 32, 8, false, MODE_STEP, EXT, UNIT>(grid, s, a, occ);
+    if (tx == 64 && ty == 4)
+        return moving ? run2d<P, 64, 4, true, MODE_STEP, EXT, UNIT>(grid, s, a, occ)
+                      : run2d<P, 64, 4, false, MODE_STEP, EXT, UNIT>(grid, s, a, occ);
+    if (tx == 32 && ty == 16)
+        return moving ? run2d<P, 32, 16, true, MODE_STEP, EXT, UNIT>(grid, s, a, occ)
+                      : run2d<P, 32, 16, false, MODE_STEP, EXT, UNIT>(grid, s, a, occ);
+    if constexpr (P::id == 0) {
+        if (tx == 16 && ty == 8)
+            return moving ? run2d<P, 16, 8, true, MODE_STEP, EXT, UNIT>(grid, s, a, occ)
+                          : run2d<P, 16, 8, false, MODE_STEP, EXT, UNIT>(grid, s, a, occ);
+    }
+    return false;
+}
+
 template <class P, bool EXT>
-static bool dispatch2d_single(int tx, int ty, bool moving, int mode, int grid, cudaStream_t s,
+static bool dispatch2d_single(int tx, int ty, bool moving, bool unit, int mode, int grid, cudaStream_t s,
                               const StepArgs &a, int *occ)
 {
     if (mode == MODE_MACROS) {
@@ -159,16 +179,8 @@ static bool dispatch2d_single(int tx, int ty, bool moving, int mode, int grid, c
                           : run2d<P, 32, 8, false, MODE_MACROS, EXT>(grid, s, a, occ);
         return false;
     }
-    if (tx == 32 && ty == 8)
-        return moving ? run2d<P, 32, 8, true, MODE_STEP, EXT>(grid, s, a, occ)
-                      : run2d<P, 32, 8, false, MODE_STEP, EXT>(grid, s, a, occ);
-    if (tx == 64 && ty == 4)
-        return moving ? run2d<P, 64, 4, true, MODE_STEP, EXT>(grid, s, a, occ)
-                      : run2d<P, 64, 4, false, MODE_STEP, EXT>(grid, s, a, occ);
-    if (tx == 32 && ty == 16)
-        return moving ? run2d<P, 32, 16, true, MODE_STEP, EXT>(grid, s, a, occ)
-                      : run2d<P, 32, 16, false, MODE_STEP, EXT>(grid, s, a, occ);
-    return false;
+    return unit ? dispatch2d_step<P, EXT, true>(tx, ty, moving, grid, s, a, occ)
+                : dispatch2d_step<P, EXT, false>(tx, ty, moving, grid, s, a, occ);
 }
 
 template <class P>
@@ -184,8 +196,8 @@ static bool dispatch2d(int tx, int ty, bool moving, int mode, int grid, cudaStre
         return !wall && !ext && !cac && dispatch2d_stage<P>(tx, ty, moving, grid, s, a, occ);
     if (mode == MODE_STEP_STRIP || mode == MODE_FILL_GHOSTS)
         return dispatch2d_strip<P>(tx, moving, cac, unit, wall, mode == MODE_FILL_GHOSTS, grid, s, a, occ);
-    return ext ? dispatch2d_single<P, true>(tx, ty, moving, mode, grid, s, a, occ)
-               : dispatch2d_single<P, false>(tx, ty, moving, mode, grid, s, a, occ);
+    return ext ? dispatch2d_single<P, true>(tx, ty, moving, unit, mode, grid, s, a, occ)
+               : dispatch2d_single<P, false>(tx, ty, moving, unit, mode, grid, s, a, occ);
 }
 
 }  // namespace pf

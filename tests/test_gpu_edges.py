@@ -124,3 +124,21 @@ def test_moving_3d_near_lists(pf, precision, shape, walls):
         pg, po = g.particle(k), o.particle(k)
         assert np.abs(np.array(pg["x"]) - np.array(po.x)).max() <= 1e-6 * max(shape), k
         assert np.abs(np.array(pg["F"]) - np.array(po.F)).max() <= (1e-11 if precision == "p64" else 2e-3) * F, k
+
+
+# 16 x 8 half tiles (few cells) and 32 x 8 tiles (one per SM), ragged in both directions; solid-free
+# frames, frames at a solid's rim, walls; unit rates (s0 free) and general ones
+@pytest.mark.parametrize("shape,walls,solid,unit", [
+    ((128, 128), False, False, True), ((7, 33), False, False, True), ((9, 17), True, True, True),
+    ((61, 50), False, True, True), ((151, 250), False, True, True), ((40, 47), True, True, False),
+])
+def test_fp64_2d_unit_and_half_tiles(pf, shape, walls, solid, unit):
+    """The FP64 2D step (unit-rate collisions, shared divisions, half tiles): the oracle at 1e-12."""
+    c = W.small_case(shape, seed=8, solid=solid, theta_deg=65.0, u_amp=0.01, rho_ratio=3.0, mu_ratio=2.0)
+    c["params"].update(s0=1.6, solid_eps=1e-3)
+    if not unit:
+        c["params"].update(s1=0.9, s2=1.1, s3=1.2, s4=0.8, eta=0.3)
+    g, o = _pair(pf, c, 6, precision="p64", walls=walls)
+    gm, om = g.macros(), o.macros()
+    for k in ("phi", "u", "P", "mu"):
+        assert np.abs(gm[k] - om[k]).max() <= 1e-12 * max(np.abs(om[k]).max(), 1e-3), k
