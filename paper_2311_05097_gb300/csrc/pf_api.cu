@@ -492,6 +492,7 @@ struct Engine {
     // tables of the macro kernel, built on first use
     double *d_macro = nullptr;
     DomainDev *d_mdoms = nullptr;
+    MacroOut *d_mouts = nullptr;             // pf_batch_get_macros_all: every domain's outputs
     // pf_batch_init_all / pf_batch_get_macros_all: host copies run on a copy
     // stream beside the engine's stream (the input copies of later domains
     // overlap the init kernels of earlier ones; the readback of a domain
@@ -505,7 +506,6 @@ struct Engine {
     cudaEvent_t ev_in = nullptr, ev_start = nullptr, ev_k[KS] = {}, ev_c[PIPE] = {};
     int nslots = 0;                          // macro buffers in rotation (d_macro and d_macro_x)
     double *d_macro_x[PIPE - 1] = {};
-    DomainDev *d_mdoms_x[PIPE - 1] = {};
     int *d_mtdom = nullptr;
     int2 *d_mtxy = nullptr;
     std::vector<int> mbase, mcount;
@@ -582,9 +582,9 @@ static void engine_free(Engine &E)
     staging_release(E.staging);
     if (E.d_macro) cudaFree(E.d_macro);
     if (E.d_mdoms) cudaFree(E.d_mdoms);
+    if (E.d_mouts) cudaFree(E.d_mouts);
     for (int k = 0; k < Engine::PIPE - 1; ++k) {
         if (E.d_macro_x[k]) cudaFree(E.d_macro_x[k]);
-        if (E.d_mdoms_x[k]) cudaFree(E.d_mdoms_x[k]);
     }
     for (int k = 0; k < Engine::KS - 1; ++k)
         if (E.kstream[k]) cudaStreamDestroy(E.kstream[k]);
@@ -637,9 +637,9 @@ static int occupancy_any(const Engine &E, int tx, int ty, int mode);
 // chunks pay where the tiles would not fill the SMs and long ones where they do
 // many times over.  131 x 100 x 90 (FP32): 191 us per step at 32 planes a chunk,
 // 118 at 12; 256^3 (16-bit): 1109 us at 8, 1065 at 16, 1118 at 22.
-static int zchunk3d(const Engine &E, int tx, int ty)
+static int zchunk3d(const Engine &E, int tx, int ty, int mode = MODE_STEP)
 {
-    const int chunks = pair3d(E) ? 2 : 1, occ = std::max(1, occupancy_any(E, tx, ty, MODE_STEP));
+    const int chunks = mode == MODE_STEP && pair3d(E) ? 2 : 1, occ = std::max(1, occupancy_any(E, tx, ty, mode));
     const double full = 0.55 + 0.45 * occ;
     int best = 1;
     double tbest = 1e300;
@@ -1338,15 +1338,11 @@ static int engine_sync(Engine &E)
     return flags_rc(E, flag);
 }
 
-// tile tables and output buffer of the macroscopic pass, built once
+// tile tables of the macroscopic pass, built once
 static int engine_macro_tables(Engine &E)
 {
     if (E.d_mdoms) return PF_OK;
     const int nd = (int)E.mem.size();
-    long long nmax = 0;
-    for (auto &m : E.mem) nmax = std::max(nmax, (long long)m.d.nx * m.d.ny * m.d.nz);
-    // planes: phi, rho, u (dim), P, mu, phi0, W, V, and the interface normal (dim)
-    CK(cudaMalloc(&E.d_macro, sizeof(double) * (size_t)(7 + 2 * E.dim) * nmax));
     int mtx = 32, mty = 8;
     if (E.dim == 3) tile_shape3d(E.prec, &mtx, &mty);
     // build_tiles writes the tiling into the DomainDev it is given: tile copies
@@ -1355,47 +1351,93 @@ static int engine_macro_tables(Engine &E)
     for (auto &c : copies) ds.push_back(&c);
     std::vector<int> tdom;
     std::vector<int2> txy;
-    build_tiles(ds, mtx, mty, tdom, txy);
+    // (3D: z chunks sized to the chip as for the step: 131 x 100 x 90 had 32 planes
+    // in each of 195 tiles)
+    build_tiles(ds, mtx, mty, tdom, txy, E.dim == 3 ? zchunk3d(E, mtx, mty, MODE_MACROS) : 1);
     std::vector<DomainDev> dd(nd);
     E.mbase.assign(nd, 0);
     E.mcount.assign(nd, 0);
     for (int k = 0; k < nd; ++k) {
         dd[k] = copies[k].d;
-        dd[k].macro = E.d_macro;
         E.mbase[k] = dd[k].tile_base;
         E.mcount[k] = dd[k].tiles_x * dd[k].tiles_y * dd[k].tiles_z;
     }
-    CK(cudaMalloc(&E.d_mdoms, sizeof(DomainDev) * nd));
-    CK(cudaMalloc(&E.d_mtdom, sizeof(int) * tdom.size()));
-    CK(cudaMalloc(&E.d_mtxy, sizeof(int2) * txy.size()));
-    CK(cudaMemcpy(E.d_mdoms, dd.data(), sizeof(DomainDev) * nd, cudaMemcpyHostToDevice));
+    if (!E.d_mtdom) CK(cudaMalloc(&E.d_mtdom, sizeof(int) * tdom.size()));
+    if (!E.d_mtxy) CK(cudaMalloc(&E.d_mtxy, sizeof(int2) * txy.size()));
     CK(cudaMemcpy(E.d_mtdom, tdom.data(), sizeof(int) * tdom.size(), cudaMemcpyHostToDevice));
     CK(cudaMemcpy(E.d_mtxy, txy.data(), sizeof(int2) * txy.size(), cudaMemcpyHostToDevice));
+    DomainDev *dev = nullptr;
+    CK(cudaMalloc(&dev, sizeof(DomainDev) * nd));
+    E.d_mdoms = dev;
+    CK(cudaMemcpy(E.d_mdoms, dd.data(), sizeof(DomainDev) * nd, cudaMemcpyHostToDevice));
+    return PF_OK;
+}
+
+// bytes of one macro buffer (largest domain): phi, rho, u (dim), P, mu, phi0, W, V,
+// and the interface normal (dim)
+static size_t macro_bytes(const Engine &E)
+{
+    long long nmax = 0;
+    for (auto &m : E.mem) nmax = std::max(nmax, (long long)m.d.nx * m.d.ny * m.d.nz);
+    return sizeof(double) * (size_t)(7 + 2 * E.dim) * nmax;
+}
+
+// the planes of domain i in a macro buffer
+static MacroOut macro_planes(const Engine &E, int i, double *b)
+{
+    const DomainDev &d = E.mem[i].d;
+    const long long N = (long long)d.nx * d.ny * d.nz;
+    double *q = b + (2 + E.dim) * N;
+    return {b, b + N, b + 2 * N, q, q + N, q + 2 * N, q + 3 * N, q + 4 * N};
+}
+
+static int engine_macro_buffer(Engine &E)
+{
+    if (!E.d_macro) CK(cudaMalloc(&E.d_macro, macro_bytes(E)));
     return PF_OK;
 }
 
 // the macro buffers of pf_batch_get_macros_all beyond the first (as many as
-// fit in 256 MiB together, 0 .. PIPE - 1) and their domain tables (the first
-// table with each domain's macro pointer moved to the buffer)
+// fit in 256 MiB together, 0 .. PIPE - 1)
 static int engine_macro_slots(Engine &E)
+{
+    int rc = engine_macro_buffer(E);
+    if (rc) return rc;
+    if (E.nslots) return PF_OK;
+    const size_t bytes = macro_bytes(E);
+    const int extra = (int)std::min<size_t>(Engine::PIPE - 1, ((size_t)256 << 20) / bytes);
+    for (int k = 0; k < extra; ++k)
+        if (!E.d_macro_x[k]) CK(cudaMalloc(&E.d_macro_x[k], bytes));
+    E.nslots = 1 + extra;
+    return PF_OK;
+}
+
+// queue the macroscopic pass of domain i (into out), or of every domain (i < 0:
+// into E.d_mouts)
+static int engine_macros_to(Engine &E, int i, const MacroOut &out)
 {
     int rc = engine_macro_tables(E);
     if (rc) return rc;
-    if (E.nslots) return PF_OK;
+    int mtx = 32, mty = 8;
+    if (E.dim == 3) tile_shape3d(E.prec, &mtx, &mty);
     const int nd = (int)E.mem.size();
-    long long nmax = 0;
-    for (auto &m : E.mem) nmax = std::max(nmax, (long long)m.d.nx * m.d.ny * m.d.nz);
-    const size_t bytes = sizeof(double) * (size_t)(7 + 2 * E.dim) * nmax;
-    const int extra = (int)std::min<size_t>(Engine::PIPE - 1, ((size_t)256 << 20) / bytes);
-    std::vector<DomainDev> dd(nd);
-    CK(cudaMemcpy(dd.data(), E.d_mdoms, sizeof(DomainDev) * nd, cudaMemcpyDeviceToHost));
-    for (int k = 0; k < extra; ++k) {
-        CK(cudaMalloc(&E.d_macro_x[k], bytes));
-        for (auto &d : dd) d.macro = E.d_macro_x[k];
-        CK(cudaMalloc(&E.d_mdoms_x[k], sizeof(DomainDev) * nd));
-        CK(cudaMemcpy(E.d_mdoms_x[k], dd.data(), sizeof(DomainDev) * nd, cudaMemcpyHostToDevice));
-    }
-    E.nslots = 1 + extra;
+    StepArgs a{};
+    a.doms = E.d_mdoms;
+    a.tile_dom = E.d_mtdom + (i < 0 ? 0 : E.mbase[i]);
+    a.tile_xy = E.d_mtxy + (i < 0 ? 0 : E.mbase[i]);
+    a.ntiles = i < 0 ? E.mbase[nd - 1] + E.mcount[nd - 1] : E.mcount[i];
+    a.par = E.par;
+    a.parts = E.d_parts;
+    a.np = E.np;
+    a.partials = nullptr;
+    a.flags = E.d_flags;
+    a.wv = E.wv;
+    a.mout = out;
+    a.mouts = i < 0 ? E.d_mouts : nullptr;
+    const int grid = std::min<int>(a.ntiles, E.nsm * 4);
+    if (!launch_any(E, mtx, mty, MODE_MACROS, grid, a))
+        return fail(PF_EINVAL, "macro kernel not built");
+    CK(cudaGetLastError());
     return PF_OK;
 }
 
@@ -1403,26 +1445,58 @@ static int engine_macro_slots(Engine &E)
 // E.d_macro_x[slot - 1]; valid until the next macroscopic pass into it)
 static int engine_macros(Engine &E, int i, int slot = 0)
 {
-    int rc = engine_macro_tables(E);
+    int rc = engine_macro_buffer(E);
     if (rc) return rc;
-    int mtx = 32, mty = 8;
-    if (E.dim == 3) tile_shape3d(E.prec, &mtx, &mty);
-    StepArgs a{};
-    a.doms = slot ? E.d_mdoms_x[slot - 1] : E.d_mdoms;
-    a.tile_dom = E.d_mtdom + E.mbase[i];
-    a.tile_xy = E.d_mtxy + E.mbase[i];
-    a.ntiles = E.mcount[i];
-    a.par = E.par;
-    a.parts = E.d_parts;
-    a.np = E.np;
-    a.partials = nullptr;
-    a.flags = E.d_flags;
-    a.wv = E.wv;
-    const int grid = std::min<int>(E.mcount[i], E.nsm * 4);
-    if (!launch_any(E, mtx, mty, MODE_MACROS, grid, a))
-        return fail(PF_EINVAL, "macro kernel not built");
-    CK(cudaGetLastError());
-    return PF_OK;
+    return engine_macros_to(E, i, macro_planes(E, i, slot ? E.d_macro_x[slot - 1] : E.d_macro));
+}
+
+// Arrays the macroscopic pass may write in place of copies: 8-byte aligned, each
+// inside one allocation of this device, no two overlapping (else the pass goes to
+// the engine's buffer and copies follow, with the copies' own errors).
+struct OutRange {
+    const void *p;
+    size_t bytes;
+};
+static bool direct_outputs(std::vector<OutRange> &r)
+{
+    typedef CUresult (*RangeFn)(CUdeviceptr *, size_t *, CUdeviceptr);
+    static const RangeFn range_of = [] {
+        void *f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 3020, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess)
+            f = nullptr;
+        return reinterpret_cast<RangeFn>(f);
+    }();
+    int dev = 0;
+    if (!range_of || cudaGetDevice(&dev) != cudaSuccess) return false;
+    for (const OutRange &o : r) {
+        cudaPointerAttributes at{};
+        CUdeviceptr base = 0;
+        size_t size = 0;
+        const CUdeviceptr v = reinterpret_cast<CUdeviceptr>(o.p);
+        if (v % 8 || cudaPointerGetAttributes(&at, o.p) != cudaSuccess || at.type != cudaMemoryTypeDevice ||
+            at.device != dev || range_of(&base, &size, v) != CUDA_SUCCESS || v + o.bytes > base + size) {
+            (void)cudaGetLastError();
+            return false;
+        }
+    }
+    std::sort(r.begin(), r.end(), [](const OutRange &a, const OutRange &b) { return a.p < b.p; });
+    for (size_t k = 1; k < r.size(); ++k)
+        if (static_cast<const char *>(r[k - 1].p) + r[k - 1].bytes > r[k].p) return false;
+    return true;
+}
+
+// the fields of domain i wanted by the caller, and their ranges
+static MacroOut wanted(const Engine &E, int i, double *phi, double *rho, double *u, double *P, double *mu,
+                       std::vector<OutRange> &r)
+{
+    const DomainDev &d = E.mem[i].d;
+    const size_t N = sizeof(double) * (size_t)d.nx * d.ny * d.nz;
+    double *f[5] = {phi, rho, u, P, mu};
+    for (int k = 0; k < 5; ++k)
+        if (f[k]) r.push_back({f[k], k == 2 ? E.dim * N : N});
+    return {phi, rho, u, P, mu, nullptr, nullptr, nullptr};
 }
 
 // the macroscopic pass of domain i and the copies of the requested fields,
@@ -1430,6 +1504,12 @@ static int engine_macros(Engine &E, int i, int slot = 0)
 static int engine_queue_macros(Engine &E, int i, double *phi, double *rho, double *u, double *P, double *mu,
                                int where)
 {
+    if (where == PF_DEVICE) {
+        // written by the pass itself: no buffer, no copies (512^2: 54 us a call with them)
+        std::vector<OutRange> r;
+        const MacroOut out = wanted(E, i, phi, rho, u, P, mu, r);
+        if (direct_outputs(r)) return engine_macros_to(E, i, out);
+    }
     int rc = engine_macros(E, i);
     if (rc) return rc;
     const DomainMem &m = E.mem[i];
@@ -1452,12 +1532,17 @@ static int engine_get_macros(Engine &E, int i, double *phi, double *rho, double 
     PfRange range("pf_get_macros");
     if (where != PF_HOST && where != PF_DEVICE) return fail(PF_EINVAL, "where must be PF_HOST or PF_DEVICE");
     if (!E.inited[i]) return fail(PF_ESTATE, "pf_get_macros before pf_init_fields");
-    int rc = engine_sync(E);
-    if (rc && rc != PF_ENUMERIC) return rc;
-    rc = engine_queue_macros(E, i, phi, rho, u, P, mu, where);
+    if (E.sticky) return E.sticky;
+    // queued behind the steps, one wait: the steps' flags come with it
+    int rc = engine_queue_macros(E, i, phi, rho, u, P, mu, where);
+    int flag = 0;
+    const cudaError_t ce = cudaMemcpyAsync(&flag, E.d_flags, sizeof(int), cudaMemcpyDeviceToHost, E.stream);
+    const int wrc = engine_wait(E);
+    if (wrc) return wrc;
     if (rc) return rc;
-    CK(cudaStreamSynchronize(E.stream));
-    return PF_OK;
+    CK(ce);
+    rc = flags_rc(E, flag);
+    return rc == PF_ENUMERIC ? PF_OK : rc;
 }
 
 // interface normal n = grad phi / |grad phi| of domain i (0 where |grad phi|^2 <= 1e-24)
@@ -2038,6 +2123,30 @@ extern "C" int pf_batch_get_macros_all(pf_batch *b, double *const *phi, double *
     if (where != PF_HOST && where != PF_DEVICE) return fail(PF_EINVAL, "where must be PF_HOST or PF_DEVICE");
     for (size_t i = 0; i < E.mem.size(); ++i)
         if (!E.inited[i]) return fail(PF_ESTATE, "pf_batch_get_macros_all before every domain is initialised");
+    if (where == PF_DEVICE) {
+        // one pass over every domain's tiles writes the caller's arrays: a sweep of 64
+        // domains took 64 passes and 192 copies, 1.07 ms
+        if (E.sticky) return E.sticky;
+        const size_t nd = E.mem.size();
+        std::vector<OutRange> r;
+        std::vector<MacroOut> tab(nd);
+        for (size_t i = 0; i < nd; ++i)
+            tab[i] = wanted(E, (int)i, phi ? phi[i] : nullptr, rho ? rho[i] : nullptr, u ? u[i] : nullptr,
+                            P ? P[i] : nullptr, mu ? mu[i] : nullptr, r);
+        if (direct_outputs(r)) {
+            if (!E.d_mouts) CK(cudaMalloc(&E.d_mouts, sizeof(MacroOut) * nd));
+            CK(cudaMemcpyAsync(E.d_mouts, tab.data(), sizeof(MacroOut) * nd, cudaMemcpyHostToDevice, E.stream));
+            int rc = engine_macros_to(E, -1, MacroOut{});
+            int flag = 0;
+            const cudaError_t ce = cudaMemcpyAsync(&flag, E.d_flags, sizeof(int), cudaMemcpyDeviceToHost, E.stream);
+            const int wrc = engine_wait(E);
+            if (wrc) return wrc;
+            if (rc) return rc;
+            CK(ce);
+            rc = flags_rc(E, flag);
+            return rc == PF_ENUMERIC ? PF_OK : rc;
+        }
+    }
     int rc = engine_sync(E);
     if (rc && rc != PF_ENUMERIC) return rc;
     rc = engine_macro_slots(E);

@@ -216,7 +216,7 @@ struct DomainDev {
     void *aux[2];    // lagged fields
     void *phi0;      // fixed indicator (3D in FP32 arithmetic: then a plane for phi of the step
                      // under way, k_phi3d)
-    double *macro;   // MODE_MACROS output: phi, rho, u(dim), P, mu, phi0 (double)
+    double *macro;   // the planes phi, rho, u(dim), P, mu, phi0, W, V the diagnostics read (double)
     int tile_base;   // index of this domain's first tile in the partial-sum table
     int tiles_x, tiles_y, tiles_z;
     int zc;                // 3D: planes per z chunk of a tile (the last chunk may be shorter);
@@ -250,6 +250,12 @@ __device__ __forceinline__ const KUnit<float> &kunit<float>(const DomainDev &d) 
 template <>
 __device__ __forceinline__ const KUnit<double> &kunit<double>(const DomainDev &d) { return d.ud; }
 
+// Where the macroscopic pass writes one domain's fields (null: not wanted); u
+// holds dim planes of N cells.
+struct MacroOut {
+    double *phi, *rho, *u, *P, *mu, *phi0, *W, *V;
+};
+
 // Arguments of the step / macro kernels (2D and 3D).
 struct StepArgs {
     const DomainDev *doms;
@@ -273,6 +279,8 @@ struct StepArgs {
     const int4 *items;              // strip kernel: work items (domain, x0, first row, end row)
     int nitems;
     const void *strip_maps;         // strip kernel: the tensor maps of every domain (128 bytes each)
+    MacroOut mout;                  // MODE_MACROS: the outputs of the only domain of the launch,
+    const MacroOut *mouts;          // or, when not null, those of every domain
     const DomainDev *dom1;          // host copy of the only domain of the launch (3D two-cells step), or null
 };
 

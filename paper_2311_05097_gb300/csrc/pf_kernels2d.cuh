@@ -765,17 +765,18 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY, UNIT && 
                 const long long o = (long long)gy * nx + gx;
                 double phv = (double)phi;
                 if constexpr (P::MIX) phv = double_of_fixed(racc);
-                Dm.macro[0 * N + o] = phv;
-                Dm.macro[1 * N + o] = (double)rho;
-                Dm.macro[2 * N + o] = (double)ux;
-                Dm.macro[3 * N + o] = (double)uy;
-                Dm.macro[4 * N + o] = (double)Pr;
-                Dm.macro[5 * N + o] = (double)mu;
-                Dm.macro[6 * N + o] = (double)phi0;
+                const MacroOut mo = A.mouts ? A.mouts[A.tile_dom[t]] : A.mout;
+                if (mo.phi) mo.phi[o] = phv;
+                if (mo.rho) mo.rho[o] = (double)rho;
+                if (mo.u) mo.u[o] = (double)ux;
+                if (mo.u) mo.u[N + o] = (double)uy;
+                if (mo.P) mo.P[o] = (double)Pr;
+                if (mo.mu) mo.mu[o] = (double)mu;
+                if (mo.phi0) mo.phi0[o] = (double)phi0;
                 if constexpr (MOVING) {
                     if (A.wv) {
-                        Dm.macro[7 * N + o] = (double)s_W[hy][hx];
-                        Dm.macro[8 * N + o] = (double)s_V[hy][hx];
+                        if (mo.W) mo.W[o] = (double)s_W[hy][hx];
+                        if (mo.V) mo.V[o] = (double)s_V[hy][hx];
                     }
                 }
             }

@@ -928,17 +928,18 @@ __global__ void __launch_bounds__(TX *TY, (sizeof(typename P::real) == 4 && !MOV
                     const long long o = ((long long)z * ny + gy) * nx + gx;
                     double phv = (double)phi;
                     if constexpr (P::MIX) phv = double_of_fixed(rs[id] + fix24_to_rest(sold, p.klog2[0]));
-                    Dm.macro[0 * N + o] = phv;
-                    Dm.macro[1 * N + o] = (double)rho;
-                    Dm.macro[2 * N + o] = (double)ux;
-                    Dm.macro[3 * N + o] = (double)uy;
-                    Dm.macro[4 * N + o] = (double)uz;
-                    Dm.macro[5 * N + o] = (double)Pr;
-                    Dm.macro[6 * N + o] = (double)mu;
-                    Dm.macro[7 * N + o] = (double)phi0;
+                    const MacroOut mo = A.mouts ? A.mouts[A.tile_dom[t]] : A.mout;
+                    if (mo.phi) mo.phi[o] = phv;
+                    if (mo.rho) mo.rho[o] = (double)rho;
+                    if (mo.u) mo.u[o] = (double)ux;
+                    if (mo.u) mo.u[N + o] = (double)uy;
+                    if (mo.u) mo.u[2 * N + o] = (double)uz;
+                    if (mo.P) mo.P[o] = (double)Pr;
+                    if (mo.mu) mo.mu[o] = (double)mu;
+                    if (mo.phi0) mo.phi0[o] = (double)phi0;
                     if (MOVING && A.wv) {
-                        Dm.macro[8 * N + o] = (double)s_W[wrap_idx(z, 5) * FP + hy * FX + hx];
-                        Dm.macro[9 * N + o] = (double)s_V[wrap_idx(z, 5) * FP + hy * FX + hx];
+                        if (mo.W) mo.W[o] = (double)s_W[wrap_idx(z, 5) * FP + hy * FX + hx];
+                        if (mo.V) mo.V[o] = (double)s_V[wrap_idx(z, 5) * FP + hy * FX + hx];
                     }
                 }
                 continue;

@@ -142,3 +142,40 @@ def test_fp64_2d_unit_and_half_tiles(pf, shape, walls, solid, unit):
     gm, om = g.macros(), o.macros()
     for k in ("phi", "u", "P", "mu"):
         assert np.abs(gm[k] - om[k]).max() <= 1e-12 * max(np.abs(om[k]).max(), 1e-3), k
+
+
+@pytest.mark.parametrize("shapes,precision,walls", [
+    ([(7, 9), (33, 40), (64, 70)], "p64", True), ([(50, 36), (8, 130)], "fp16", False), ([(5, 6, 33), (40, 9, 8)], "p32", True),
+])
+def test_device_outputs_equal_host_ones(pf, shapes, precision, walls):
+    """Fields written by the pass into the caller's device arrays, arrays that it may not write (overlapping
+    ones: copies), fields left out, and the host's copies: the same bits."""
+    import ctypes as C
+    import torch
+    cases = [W.small_case(s, seed=k, solid=min(s) > 6, u_amp=0.01) for k, s in enumerate(shapes)]
+    b = pf.Batch(shapes, [c["params"] for c in cases], precision=precision, walls_y=walls)
+    b.init_all([c["phi0"] for c in cases], [c["phi"] for c in cases], [c["u"] for c in cases])
+    b.step(3)
+    host = b.macros_all()
+    dim, keys = len(shapes[0]), ("phi", "rho", "u", "P", "mu")
+    for left_out, shared in ((None, False), ("rho", False), (None, True)):
+        bufs, tables = [], []
+        for s in shapes:
+            N = int(np.prod(s))
+            one = torch.full(((4 + dim) * N + 1,), float("nan"), dtype=torch.float64, device="cuda")
+            at, o = 1, {}
+            for k in keys:
+                o[k] = one[at:at + (dim if k == "u" else 1) * N]
+                at += 0 if shared and k == "phi" else o[k].numel()  # (shared: rho over phi)
+            bufs.append(o)
+        for k in keys:
+            t = (C.c_void_p * len(shapes))(*[None if k == left_out else o[k].data_ptr() for o in bufs])
+            tables.append(C.cast(t, C.c_void_p))
+        assert pf.load().pf_batch_get_macros_all(b._h, *tables, pf.PF_DEVICE) == pf.PF_OK
+        for i, o in enumerate(bufs):
+            for k in keys:
+                got = o[k].cpu().numpy()
+                if k == left_out:
+                    assert np.isnan(got).all()
+                elif not (shared and k == "phi"):
+                    assert np.array_equal(got, np.asarray(host[i][k]).reshape(-1)), (i, k)
