@@ -43,6 +43,65 @@ __device__ __forceinline__ float rcp_fast(float a)
 }
 __device__ __forceinline__ F2 rcp2(F2 a) { return mk2(rcp_fast(a.v.x), rcp_fast(a.v.y)); }
 
+// two 16-bit values as one 32-bit word (a in the low half: the lower address)
+template <class S>
+__device__ __forceinline__ uint32_t pack2(S a, S b);
+template <>
+__device__ __forceinline__ uint32_t pack2<__half>(__half a, __half b)
+{
+    return (uint32_t)__half_as_ushort(a) | ((uint32_t)__half_as_ushort(b) << 16);
+}
+template <>
+__device__ __forceinline__ uint32_t pack2<__nv_bfloat16>(__nv_bfloat16 a, __nv_bfloat16 b)
+{
+    return (uint32_t)__bfloat16_as_ushort(a) | ((uint32_t)__bfloat16_as_ushort(b) << 16);
+}
+
+// two FP32 values rounded to the 16-bit storage type as one 32-bit word (one
+// conversion instruction for both), and back
+template <class S>
+__device__ __forceinline__ uint32_t cvt_pair(F2 v);
+template <>
+__device__ __forceinline__ uint32_t cvt_pair<__half>(F2 v)
+{
+    const __half2 h = __float22half2_rn(v.v);
+    return *reinterpret_cast<const uint32_t *>(&h);
+}
+template <>
+__device__ __forceinline__ uint32_t cvt_pair<__nv_bfloat16>(F2 v)
+{
+    const __nv_bfloat162 h = __float22bfloat162_rn(v.v);
+    return *reinterpret_cast<const uint32_t *>(&h);
+}
+template <class S>
+__device__ __forceinline__ F2 uncvt_pair(uint32_t w);
+template <>
+__device__ __forceinline__ F2 uncvt_pair<__half>(uint32_t w)
+{
+    return {__half22float2(*reinterpret_cast<const __half2 *>(&w))};
+}
+template <>
+__device__ __forceinline__ F2 uncvt_pair<__nv_bfloat16>(uint32_t w)
+{
+    return {__bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&w))};
+}
+// a 16-bit value from its bits
+template <class S>
+__device__ __forceinline__ S half_of(unsigned short b);
+template <>
+__device__ __forceinline__ __half half_of<__half>(unsigned short b) { return __ushort_as_half(b); }
+template <>
+__device__ __forceinline__ __nv_bfloat16 half_of<__nv_bfloat16>(unsigned short b) { return __ushort_as_bfloat16(b); }
+
+// bit pattern of FIX24_LIMIT (8.0) in the 16-bit type: |v| < 8 exactly when
+// the magnitude bits of v are below it (NaN and infinity are not)
+template <class S>
+constexpr uint32_t fix24_limit_bits();
+template <>
+constexpr uint32_t fix24_limit_bits<__half>() { return 0x4800u; }
+template <>
+constexpr uint32_t fix24_limit_bits<__nv_bfloat16>() { return 0x4100u; }
+
 // Column values a[y - 1 .. y + 2][x] of a shared array, as the pairs of the
 // stencils of rows (y, y + 1).
 template <int W>
@@ -423,12 +482,12 @@ __device__ __forceinline__ void pair_physics(int phase_model, const KParams<floa
 // order parameter (checked per domain).  MU0: the simulation holds free
 // particles, so the force carries mu_phi0 grad phi0 (Eq. 19) of the fixed
 // solids too (the tiles this kernel gets are out of every particle's reach).
-template <class P, int FX, int WX, bool CAC = false, bool MU0 = false>
+template <class P, int FX, int WX, bool CAC = false, bool MU0 = false, bool UNIT = false>
 __device__ __forceinline__ void pair_cells(const StepArgs &A, const DevParams &p, const KParams<float> &kp,
                                            const float (*s_phi)[FX], const float (*s_p0)[FX],
                                            const float (*s_mu)[WX], const float (*s_w)[WX], int hx, int hy,
                                            int wx, int wy, F2 phi, F2 (&f1)[9],
-                                           const typename P::store (&f2raw)[2][9],
+                                           const typename P::store (&f2raw)[2][9], const uint32_t (&f2w)[9],
                                            const typename P::aux (&lag)[2][5],
                                            const long long (&racc)[2], const int (&id)[2], bool valid0, bool valid1, typename P::store *fd,
                                            long long *rd, typename P::aux *ad, int plane)
@@ -452,18 +511,61 @@ __device__ __forceinline__ void pair_cells(const StepArgs &A, const DevParams &p
     const F2 isc2v = mk2(kp.inv_scale[1]);
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
-        const F2 v = P::MIX ? mk2(stored_to_float<ST>(f2raw[0][i]), stored_to_float<ST>(f2raw[1][i]))
-                            : mk2(Conv<P>::ld(f2raw[0][i], 1.0f), Conv<P>::ld(f2raw[1][i], 1.0f));
-        f2[i] = P::MIX ? v * isc2v : v;
+        if constexpr (P::MIX)
+            f2[i] = uncvt_pair<ST>(f2w[i]) * isc2v;
+        else
+            f2[i] = mk2(Conv<P>::ld(f2raw[0][i], 1.0f), Conv<P>::ld(f2raw[1][i], 1.0f));
     }
     const F2 upx = mk2((float)lag[0][0], (float)lag[1][0]), upy = mk2((float)lag[0][1], (float)lag[1][1]);
     const F2 Spx = mk2((float)lag[0][2], (float)lag[1][2]), Spy = mk2((float)lag[0][3], (float)lag[1][3]);
     const F2 php = mk2((float)lag[0][4], (float)lag[1][4]);
     F2 ux, uy, Sx, Sy;
-    pair_physics<CAC, MU0>(p.phase_model, kp, phi, phi0, mu, gpx, gpy, gmx, gmy, wgx, wgy, lphi, g0x, g0y, upx, upy,
-                           Spx, Spy, php, f1, f2, ux, uy, Sx, Sy, NoEmit(), NoEmit(), MU0 && A.wv != 0, g3x, g3y);
+    pair_physics<CAC, MU0, NoEmit, NoEmit, UNIT>(p.phase_model, kp, phi, phi0, mu, gpx, gpy, gmx, gmy, wgx, wgy, lphi,
+                                                 g0x, g0y, upx, upy, Spx, Spy, php, f1, f2, ux, uy, Sx, Sy, NoEmit(),
+                                                 NoEmit(), MU0 && A.wv != 0, g3x, g3y);
 
-    // ---------------- stores (per cell) ----------------
+    // ---------------- stores ----------------
+    // 16-bit storage: both cells' values rounded by one instruction and kept as one
+    // word per population; the images of the order parameter's as in the strip step
+    [[maybe_unused]] uint32_t w1[9], w2[9];
+    if constexpr (P::MIX) {
+        const F2 sc1 = mk2(kp.scale[0]), sc2 = mk2(kp.scale[1]), s24 = mk2(16777216.0f);
+        uint32_t amax = 0u;
+#pragma unroll
+        for (int i = 1; i < 9; ++i) {
+            w1[i] = cvt_pair<ST>(f1[i] * sc1);
+            if constexpr (P::id == 3)
+                w1[i] = pack2<ST>(bf16_flush(half_of<ST>((unsigned short)(w1[i] & 0xffffu))),
+                                  bf16_flush(half_of<ST>((unsigned short)(w1[i] >> 16))));
+            amax = __vmaxu2(amax, w1[i] & 0x7fff7fffu);
+        }
+        constexpr uint32_t lim = fix24_limit_bits<ST>();
+        if ((amax & 0xffffu) >= lim || (amax >> 16) >= lim) {
+            // a value out of the images' range: saturate it in place (rare)
+            int bad[2] = {0, 0};
+#pragma unroll
+            for (int i = 1; i < 9; ++i) {
+                ST qa = half_of<ST>((unsigned short)(w1[i] & 0xffffu));
+                ST qb = half_of<ST>((unsigned short)(w1[i] >> 16));
+                fix24_sat<ST>(qa, &bad[0]);
+                fix24_sat<ST>(qb, &bad[1]);
+                w1[i] = pack2<ST>(qa, qb);
+            }
+            if ((valid0 && bad[0]) || (valid1 && bad[1])) atomicOr(A.flags, 2);
+        }
+        int snew[2] = {0, 0};
+#pragma unroll
+        for (int i = 1; i < 9; ++i) {
+            const F2 im = uncvt_pair<ST>(w1[i]) * s24;  // exact: the stored value in 2^-24 units
+            snew[0] += __float2int_rn(im.v.x);
+            snew[1] += __float2int_rn(im.v.y);
+        }
+        // exact: the sum of each cell's order-parameter populations is unchanged
+        if (valid0) rd[id[0]] = racc[0] - fix24_to_rest(snew[0], p.klog2[0]);
+        if (valid1) rd[id[1]] = racc[1] - fix24_to_rest(snew[1], p.klog2[0]);
+#pragma unroll
+        for (int i = 0; i < 9; ++i) w2[i] = cvt_pair<ST>(f2[i] * sc2);
+    }
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
         if (!(c == 0 ? valid0 : valid1)) continue;
@@ -471,25 +573,18 @@ __device__ __forceinline__ void pair_cells(const StepArgs &A, const DevParams &p
         const float phic = c == 0 ? phi.v.x : phi.v.y;
         const float uxc = c == 0 ? ux.v.x : ux.v.y, uyc = c == 0 ? uy.v.x : uy.v.y;
         if constexpr (P::MIX) {
-            const float sc1 = kp.scale[0];
-            int bad = 0, snew = 0;
+            auto half = [&](uint32_t w) { return half_of<ST>((unsigned short)(c == 0 ? w & 0xffffu : w >> 16)); };
 #pragma unroll
-            for (int i = 1; i < 9; ++i) {
-                ST q = Conv<P>::st(c == 0 ? f1[i].v.x : f1[i].v.y, sc1);
-                if constexpr (P::id == 3) q = bf16_flush(q);
-                snew += fix24_sat<ST>(q, &bad);
-                fd[i * plane + idc] = q;
-            }
-            // exact: sum of the cell's order-parameter populations is unchanged
-            rd[idc] = racc[c] - fix24_to_rest(snew, p.klog2[0]);
-            if (bad) atomicOr(A.flags, 2);
+            for (int i = 1; i < 9; ++i) fd[i * plane + idc] = half(w1[i]);
+#pragma unroll
+            for (int i = 0; i < 9; ++i) fd[(9 + i) * plane + idc] = half(w2[i]);
         } else {
 #pragma unroll
-            for (int i = 0; i < 9; ++i) fd[i * plane + idc] = Conv<P>::st(c == 0 ? f1[i].v.x : f1[i].v.y, 1.0f);
+            for (int i = 0; i < 9; ++i) {
+                fd[i * plane + idc] = Conv<P>::st(c == 0 ? f1[i].v.x : f1[i].v.y, 1.0f);
+                fd[(9 + i) * plane + idc] = Conv<P>::st(c == 0 ? f2[i].v.x : f2[i].v.y, 1.0f);
+            }
         }
-        const float sc2 = P::MIX ? kp.scale[1] : 1.0f;
-#pragma unroll
-        for (int i = 0; i < 9; ++i) fd[(9 + i) * plane + idc] = Conv<P>::st(c == 0 ? f2[i].v.x : f2[i].v.y, sc2);
         // fields of this step, read as the previous step's by the next one
         ad[0 * plane + idc] = (AX)uxc;
         ad[1 * plane + idc] = (AX)uyc;
@@ -500,15 +595,20 @@ __device__ __forceinline__ void pair_cells(const StepArgs &A, const DevParams &p
     }
 }
 
-// 256-thread pair tiles are register heavy: two resident CTAs per SM.
-template <int TX, int TYP>
+// 256-thread pair tiles are register heavy: two resident CTAs per SM; at unit
+// rates (the order parameter's populations only summed) three of 80 registers,
+// which spill 12 (FP32) to 104 bytes (16-bit) per thread and still win: the loads
+// of stage A bound the step, and a third CTA keeps more of them in flight.  Per
+// step, two and three CTAs: a sweep of 64 domains in FP16 165 and 141 us, 1024 x
+// 1000 in FP32 51.1 and 47.5, the far tiles of 1024 x 2048 (FP16) 136 and 122.
+template <int TX, int TYP, bool UNIT = false>
 constexpr int step2d_pair_min_blocks()
 {
-    return TX * TYP > 256 ? 1 : 2;
+    return TX * TYP > 256 ? 1 : (UNIT ? 3 : 2);
 }
 
-template <class P, int TX, int TYP, bool CAC, bool MU0 = false>
-__global__ void __launch_bounds__(TX *TYP, (step2d_pair_min_blocks<TX, TYP>())) k_step2d_pair(StepArgs A)
+template <class P, int TX, int TYP, bool CAC, bool MU0 = false, bool UNIT = false>
+__global__ void __launch_bounds__(TX *TYP, (step2d_pair_min_blocks<TX, TYP, UNIT>())) k_step2d_pair(StepArgs A)
 {
     using ST = typename P::store;
     using AX = typename P::aux;
@@ -606,7 +706,7 @@ __global__ void __launch_bounds__(TX *TYP, (step2d_pair_min_blocks<TX, TYP>())) 
                 const F2 v = P::MIX ? mk2(stored_to_float<ST>(q1[0][i]), stored_to_float<ST>(q1[1][i]))
                                     : mk2(Conv<P>::ld(q1[0][i], 1.0f), Conv<P>::ld(q1[1][i], 1.0f));
                 acc = acc + v;
-                f1[i] = P::MIX ? v * mk2(isc1) : v;
+                if constexpr (!UNIT) f1[i] = P::MIX ? v * mk2(isc1) : v;
             }
             if constexpr (P::MIX) {
                 f1[0] = mk2(rest_f[0], rest_f[1]);
@@ -625,6 +725,12 @@ __global__ void __launch_bounds__(TX *TYP, (step2d_pair_min_blocks<TX, TYP>())) 
                 for (int i = 1; i < 9; ++i) sold += fix24_stored<ST>(q1[c][i]);
                 racc[c] = rest_own[c] + fix24_to_rest(sold, p.klog2[0]);
             }
+        }
+        // (16-bit storage: the two cells' flow populations wait packed in one word each)
+        uint32_t f2w[9];
+        if constexpr (P::MIX) {
+#pragma unroll
+            for (int i = 0; i < 9; ++i) f2w[i] = pack2<ST>(f2raw[0][i], f2raw[1][i]);
         }
         const int hx = lx + 2, hy = ly0 + 2;
         s_phi[hy][hx] = phi.v.x;
@@ -681,7 +787,7 @@ __global__ void __launch_bounds__(TX *TYP, (step2d_pair_min_blocks<TX, TYP>())) 
         {
             const int gx = x0 + lx, gy0 = y0 + ly0;
             const bool valid0 = gx < nx && gy0 < ny, valid1 = gx < nx && gy0 + 1 < ny;
-            pair_cells<P, FX, WX, CAC, MU0>(A, p, kp, s_phi, s_p0, s_mu, s_w, hx, hy, lx + 1, ly0 + 1, phi, f1, f2raw, lag, racc,
+            pair_cells<P, FX, WX, CAC, MU0, UNIT>(A, p, kp, s_phi, s_p0, s_mu, s_w, hx, hy, lx + 1, ly0 + 1, phi, f1, f2raw, f2w, lag, racc,
                                   id, valid0, valid1, fd, rd, ad, plane);
         }
     }

@@ -331,7 +331,12 @@ __global__ void __launch_bounds__(TX *TYP, (step2d_pair_min_blocks<TX, TYP>())) 
         {
             const int gx = x0 + lx, gy0 = y0 + ly0;
             const bool valid0 = gx < nx && gy0 < ny, valid1 = gx < nx && gy0 + 1 < ny;
-            pair_cells<P, FX, WX>(A, p, kp, s_phi, s_p0, s_mu, s_w, hx, hy, lx + 1, ly0 + 1, phi, f1, f2raw, lag, racc,
+            uint32_t f2w[9];
+            if constexpr (P::MIX) {
+#pragma unroll
+                for (int i = 0; i < 9; ++i) f2w[i] = pack2<ST>(f2raw[0][i], f2raw[1][i]);
+            }
+            pair_cells<P, FX, WX>(A, p, kp, s_phi, s_p0, s_mu, s_w, hx, hy, lx + 1, ly0 + 1, phi, f1, f2raw, f2w, lag, racc,
                                   id, valid0, valid1, fd, rd, ad, plane);
         }
     }

@@ -127,65 +127,6 @@ __device__ __forceinline__ F2 lap9_hpair(const float4 (&w)[3])
     return fma2(mk2(2.0f / 3.0f), side, fma2(mk2(1.0f / 6.0f), diag, mk2(-10.0f / 3.0f) * Mc));
 }
 
-// two 16-bit values as one 32-bit word (a in the low half: the lower address)
-template <class S>
-__device__ __forceinline__ uint32_t pack2(S a, S b);
-template <>
-__device__ __forceinline__ uint32_t pack2<__half>(__half a, __half b)
-{
-    return (uint32_t)__half_as_ushort(a) | ((uint32_t)__half_as_ushort(b) << 16);
-}
-template <>
-__device__ __forceinline__ uint32_t pack2<__nv_bfloat16>(__nv_bfloat16 a, __nv_bfloat16 b)
-{
-    return (uint32_t)__bfloat16_as_ushort(a) | ((uint32_t)__bfloat16_as_ushort(b) << 16);
-}
-
-// two FP32 values rounded to the 16-bit storage type as one 32-bit word (one
-// conversion instruction for both), and back
-template <class S>
-__device__ __forceinline__ uint32_t cvt_pair(F2 v);
-template <>
-__device__ __forceinline__ uint32_t cvt_pair<__half>(F2 v)
-{
-    const __half2 h = __float22half2_rn(v.v);
-    return *reinterpret_cast<const uint32_t *>(&h);
-}
-template <>
-__device__ __forceinline__ uint32_t cvt_pair<__nv_bfloat16>(F2 v)
-{
-    const __nv_bfloat162 h = __float22bfloat162_rn(v.v);
-    return *reinterpret_cast<const uint32_t *>(&h);
-}
-template <class S>
-__device__ __forceinline__ F2 uncvt_pair(uint32_t w);
-template <>
-__device__ __forceinline__ F2 uncvt_pair<__half>(uint32_t w)
-{
-    return {__half22float2(*reinterpret_cast<const __half2 *>(&w))};
-}
-template <>
-__device__ __forceinline__ F2 uncvt_pair<__nv_bfloat16>(uint32_t w)
-{
-    return {__bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&w))};
-}
-// a 16-bit value from its bits
-template <class S>
-__device__ __forceinline__ S half_of(unsigned short b);
-template <>
-__device__ __forceinline__ __half half_of<__half>(unsigned short b) { return __ushort_as_half(b); }
-template <>
-__device__ __forceinline__ __nv_bfloat16 half_of<__nv_bfloat16>(unsigned short b) { return __ushort_as_bfloat16(b); }
-
-// bit pattern of FIX24_LIMIT (8.0) in the 16-bit type: |v| < 8 exactly when
-// the magnitude bits of v are below it (NaN and infinity are not)
-template <class S>
-constexpr uint32_t fix24_limit_bits();
-template <>
-constexpr uint32_t fix24_limit_bits<__half>() { return 0x4800u; }
-template <>
-constexpr uint32_t fix24_limit_bits<__nv_bfloat16>() { return 0x4100u; }
-
 // the lane index, read afresh where it is used (volatile: the values derived
 // from it are not hoisted out of the band loop, where they would hold
 // registers through the update)

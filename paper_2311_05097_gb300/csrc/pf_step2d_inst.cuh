@@ -25,10 +25,10 @@ static bool run2d(int grid, cudaStream_t s, const StepArgs &a, int *occ)
     return true;
 }
 
-template <class P, int TX, int TYP, bool CAC, bool MU0 = false>
+template <class P, int TX, int TYP, bool CAC, bool MU0 = false, bool UNIT = false>
 static bool run2d_pair(int grid, cudaStream_t s, const StepArgs &a, int *occ)
 {
-    auto kern = k_step2d_pair<P, TX, TYP, CAC, MU0>;
+    auto kern = k_step2d_pair<P, TX, TYP, CAC, MU0, UNIT>;
     if (occ) {
         int n = 0;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, TX * TYP, 0) != cudaSuccess) n = 0;
@@ -42,15 +42,25 @@ static bool run2d_pair(int grid, cudaStream_t s, const StepArgs &a, int *occ)
 
 // two cells per thread: tiles of tx x ty cells on tx x ty/2 threads
 template <class P>
-static bool dispatch2d_pair(int tx, int ty, bool moving, bool cac, bool mu0, int grid, cudaStream_t s,
+static bool dispatch2d_pair(int tx, int ty, bool moving, bool cac, bool mu0, bool unit, int grid, cudaStream_t s,
                             const StepArgs &a, int *occ)
 {
     if constexpr (P::id == 0) {
         return false;  // FP64 has no packed arithmetic
     } else {
         // far tiles of a particle domain: 32 x 16, Cahn-Hilliard
-        if (mu0) return tx == 32 && ty == 16 && !cac && run2d_pair<P, 32, 8, false, true>(grid, s, a, occ);
+        if (mu0) {
+            if (tx != 32 || ty != 16 || cac) return false;
+            return unit ? run2d_pair<P, 32, 8, false, true, true>(grid, s, a, occ)
+                        : run2d_pair<P, 32, 8, false, true>(grid, s, a, occ);
+        }
         if (moving) return false;
+        if (unit && !cac) {
+            if (tx == 32 && ty == 16) return run2d_pair<P, 32, 8, false, false, true>(grid, s, a, occ);
+            if (tx == 64 && ty == 8) return run2d_pair<P, 64, 4, false, false, true>(grid, s, a, occ);
+            if (tx == 32 && ty == 32) return run2d_pair<P, 32, 16, false, false, true>(grid, s, a, occ);
+            return false;
+        }
         if (tx == 32 && ty == 16)
             return cac ? run2d_pair<P, 32, 8, true>(grid, s, a, occ) : run2d_pair<P, 32, 8, false>(grid, s, a, occ);
         if (tx == 64 && ty == 8)
@@ -191,7 +201,7 @@ static bool dispatch2d(int tx, int ty, bool moving, int mode, int grid, cudaStre
     const bool wall = (mode & MODE_WALL) != 0, unit = (mode & MODE_UNIT) != 0;
     mode &= ~(MODE_EXT | MODE_CAC | MODE_MU0 | MODE_WALL | MODE_UNIT);
     // the tiled two-cells-per-thread kernels have no wall handling: refuse walled launches
-    if (mode == MODE_STEP_PAIR) return !wall && dispatch2d_pair<P>(tx, ty, moving, cac, mu0, grid, s, a, occ);
+    if (mode == MODE_STEP_PAIR) return !wall && dispatch2d_pair<P>(tx, ty, moving, cac, mu0, unit, grid, s, a, occ);
     if (mode == MODE_STEP_STAGE)
         return !wall && !ext && !cac && dispatch2d_stage<P>(tx, ty, moving, grid, s, a, occ);
     if (mode == MODE_STEP_STRIP || mode == MODE_FILL_GHOSTS)

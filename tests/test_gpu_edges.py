@@ -179,3 +179,38 @@ def test_device_outputs_equal_host_ones(pf, shapes, precision, walls):
                     assert np.isnan(got).all()
                 elif not (shared and k == "phi"):
                     assert np.array_equal(got, np.asarray(host[i][k]).reshape(-1)), (i, k)
+
+
+@pytest.mark.parametrize("shape", [(4, 5), (17, 33), (16, 64), (47, 95)])
+@pytest.mark.parametrize("precision", ["p32", "fp16", "bf16"])
+@pytest.mark.parametrize("unit", [True, False])
+def test_pair_2d_unit_rates(pf, shape, precision, unit):
+    """The tiled two-cells step at unit and general rates, tiles ragged in both directions, against the oracle:
+    a few roundings of six steps (FP32 6e-8; 16-bit movers 2^-11 and 2^-8 of sizes below 0.02)."""
+    tol = dict(p32=dict(phi=2e-6, u=1e-4), fp16=dict(phi=1e-4, u=2e-2), bf16=dict(phi=1e-3, u=0.2))[precision]
+    c = W.small_case(shape, seed=5, solid=min(shape) > 8, theta_deg=75.0, u_amp=0.01, rho_ratio=2.0, mu_ratio=2.0)
+    c["params"].update(solid_eps=0.1)
+    if not unit:
+        c["params"].update(s0=1.3, s1=0.9, s2=1.1, s3=1.2, s4=0.8, eta=0.3)
+    for cfg in ((32, 16, 1, 0), (64, 8, 1, 0)):
+        g, o = _pair(pf, c, 6, precision=precision, config=cfg)
+        gm, om = g.macros(), o.macros()
+        for k, t in tol.items():
+            assert np.abs(gm[k] - om[k]).max() <= t * max(np.abs(om[k]).max(), 1e-3), (cfg, k)
+
+
+@pytest.mark.parametrize("shapes", [[(5, 8), (9, 10)], [(61, 72), (257, 130), (8, 66)]])
+def test_tuned_strip_segments(pf, shapes):
+    """Batches whose domains are shorter than the shortest segment and longer than the longest: every candidate
+    the tuner runs computes the same update."""
+    cases = [W.small_case(s, seed=k, solid=False, u_amp=0.01) for k, s in enumerate(shapes)]
+    b = pf.Batch(shapes, [c["params"] for c in cases], precision="p32")
+    b.init_all([c["phi0"] for c in cases], [c["phi"] for c in cases], [c["u"] for c in cases])
+    b.step(256)
+    for i, c in enumerate(cases):
+        s = pf.Sim(c["shape"], precision="p32", **c["params"])
+        s.init(c["phi0"], c["phi"], c["u"])
+        s.step(256)
+        x, y = b.macros(i), s.macros()
+        # FP32 roundings of 256 steps (random: 6e-8 sqrt(256) of phi, 16 times that as the fields' bound)
+        assert np.abs(x["phi"] - y["phi"]).max() <= 2e-5, i
