@@ -9,6 +9,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <map>
+#include <queue>
 #include <mutex>
 #include <string>
 #include <tuple>
@@ -997,28 +998,73 @@ static int strip_setup(Engine &E, int seg)
         CK(cudaMemcpy(E.d_maps, maps.data(), sizeof(CUtensorMap) * maps.size(), cudaMemcpyHostToDevice));
         E.maps_ok = true;
     }
-    struct It {
-        int4 v;
-        long long cells;
-    };
-    std::vector<It> its;
+    // longest first (an item's time goes with its rows: a narrow last strip takes as
+    // long as a full one)
+    std::vector<int4> items;
     for (int i = 0; i < (int)E.mem.size(); ++i) {
         const DomainDev &d = E.mem[i].d;
         for (int ya = 0; ya < d.ny; ya += seg)
-            for (int x0 = 0; x0 < d.nx; x0 += STRIP_SW) {
-                const int yb = std::min(ya + seg, d.ny);
-                its.push_back({make_int4(i, x0, ya, yb), (long long)(yb - ya) * std::min(STRIP_SW, d.nx - x0)});
-            }
+            for (int x0 = 0; x0 < d.nx; x0 += STRIP_SW) items.push_back(make_int4(i, x0, ya, std::min(ya + seg, d.ny)));
     }
-    std::stable_sort(its.begin(), its.end(), [](const It &a, const It &b) { return a.cells > b.cells; });
-    std::vector<int4> items;
-    for (auto &t : its) items.push_back(t.v);
+    std::stable_sort(items.begin(), items.end(), [](int4 a, int4 b) { return a.w - a.z > b.w - b.z; });
     if (E.d_items) cudaFree(E.d_items);
     E.d_items = nullptr;
     E.nitems = (int)items.size();
     CK(cudaMalloc(&E.d_items, sizeof(int4) * items.size()));
     CK(cudaMemcpy(E.d_items, items.data(), sizeof(int4) * items.size(), cudaMemcpyHostToDevice));
     return PF_OK;
+}
+
+// The segment lengths worth timing: those whose items, handed out longest first,
+// finish earliest on the chip's two CTAs per SM by a count of rows (an item takes
+// its rows, in whole bands, and a prologue worth about ten).  1024 x 1024: 56 rows
+// make 304 items for 304 places, 51.1 us per step; 64 rows 256 items, 54.8 us; 48
+// rows 352 items, 73.7 us.
+static void strip_segments(const Engine &E, int *out, int n)
+{
+    static const int cand[] = {8, 12, 16, 20, 24, 28, 32, 36, 40, 48, 54, 56, 60, 64, 72, 80, 84, 96, 102, 108, 120, 128, 144, 160, 168, 192, 216, 256};
+    const int B = E.prec == PF_P32 ? 4 : 6;
+    std::vector<std::pair<long long, int>> rank;
+    int nymax = 0, before = 0;
+    for (auto &m : E.mem) nymax = std::max(nymax, m.d.ny);
+    for (int seg : cand) {
+        if (before >= nymax) break;  // (one segment per strip from there on)
+        before = seg;
+        std::map<int, long long, std::greater<int>> items;  // rows -> count
+        for (auto &m : E.mem) {
+            const long long strips = (m.d.nx + STRIP_SW - 1) / STRIP_SW;
+            if (m.d.ny / seg) items[seg] += strips * (m.d.ny / seg);
+            if (m.d.ny % seg) items[m.d.ny % seg] += strips;
+        }
+        // (equal items fill the places in rounds; the places are a heap by load)
+        std::priority_queue<long long, std::vector<long long>, std::greater<long long>> load;
+        for (int k = 0; k < 2 * E.nsm; ++k) load.push(0);
+        long long last = 0;
+        for (auto &it : items) {
+            const long long c = (it.first + B - 1) / B * B + 10;
+            long long left = it.second;
+            const long long rounds = left / (2 * E.nsm) > 4 ? left / (2 * E.nsm) - 4 : 0;
+            if (rounds) {  // whole rounds raise every place alike
+                std::priority_queue<long long, std::vector<long long>, std::greater<long long>> q;
+                while (!load.empty()) {
+                    q.push(load.top() + rounds * c);
+                    last = std::max(last, load.top() + rounds * c);
+                    load.pop();
+                }
+                load.swap(q);
+                left -= rounds * 2 * E.nsm;
+            }
+            for (; left > 0; --left) {
+                const long long v = load.top() + c;
+                load.pop();
+                load.push(v);
+                last = std::max(last, v);
+            }
+        }
+        rank.push_back({last, -seg});  // (ties: the longer segment)
+    }
+    std::sort(rank.begin(), rank.end());
+    for (int k = 0; k < n; ++k) out[k] = -rank[std::min<size_t>(k, rank.size() - 1)].second;
 }
 
 // fill the ghost columns of the buffers the next step reads, unless valid
@@ -1107,17 +1153,9 @@ static int engine_configure(Engine &E, bool tune)
                          {64, 128, 4}, {64, 192, 4}, {64, 256, 4}};
     int nshapes = (E.prec != PF_P64 && E.np == 0 && !any_walls(E)) ? 6 : 3;
     if (strip_ok(E)) {
-        // on small launches (fewer than 8 work items of 96 rows per SM) also
-        // the short segments that give every CTA slot work
-        long long items96 = 0;
-        for (auto &m : E.mem)
-            items96 += (long long)((m.d.nx + STRIP_SW - 1) / STRIP_SW) * ((m.d.ny + 95) / 96);
-        if (items96 < 8LL * E.nsm) {
-            shapes[6][1] = 8;
-            shapes[7][1] = 16;
-            shapes[8][1] = 32;
-            shapes[9][1] = 64;
-        }
+        int segs[4];
+        strip_segments(E, segs, 4);
+        for (int k = 0; k < 4; ++k) shapes[6 + k][1] = segs[k];
         if (nshapes == 3)
             for (int k = 0; k < 4; ++k)
                 for (int j = 0; j < 3; ++j) shapes[3 + k][j] = shapes[6 + k][j];
