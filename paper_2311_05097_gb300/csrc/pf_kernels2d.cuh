@@ -257,6 +257,7 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY, UNIT && 
     // cells then skip the FP64 minimum-image arithmetic)
     constexpr int PMAX = 64;
     __shared__ unsigned long long s_fast;
+    __shared__ unsigned long long s_own;  // near particles with their own contact angle
     __shared__ R s_pcx[MOVING ? PMAX : 1], s_pcy[MOVING ? PMAX : 1];
     // per near particle, in the arithmetic type: radius, reach R + cut, u_x, u_y,
     // w_z, cos(own angle) (0 without one)
@@ -278,7 +279,7 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY, UNIT && 
 
         __syncthreads();  // previous tile's shared-memory readers are done
         if constexpr (MOVING) {
-            if (tid == 0) s_near = s_fast = 0ull;
+            if (tid == 0) s_near = s_fast = s_own = 0ull;
         }
         const int wall = EXT ? Dm.wall_y : 0;
         const int nyw = wall ? 0 : ny;  // minimum image in y only without walls
@@ -332,6 +333,7 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY, UNIT && 
                     s_pv[k][3] = (R)pp.u[1];
                     s_pv[k][4] = (R)pp.w[2];
                     s_pv[k][5] = pp.own ? (R)pp.ct : R(0);
+                    if (pp.own) atomicOr(&s_own, 1ull << k);
                     // a cell of the frames farther than nx/2 from this image is at
                     // least R + cut + 1 from every image when the box is this wide
                     const double span = 2.0 * (pp.R + pcut) + 8.0;
@@ -411,18 +413,27 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY, UNIT && 
             }
             return acc;
         };
-        auto phi0_at = [&](int hx, int hy) -> R {
+        [[maybe_unused]] int any_solid = 0;  // some solid's indicator is not 0 in the cells this thread fills
+        // near particles are visited as the set bits of their mask (a test per particle
+        // of the domain and cell cost more than the indicators); hits: those whose
+        // indicator at this cell is not 0
+        auto phi0_at = [&](int hx, int hy, [[maybe_unused]] unsigned long long &hits) -> R {
             const int cx = hx + 1, cy = hy + 1;
             R v = (R)ldg(ph0 + s_gy[cy] + s_gx[cx]);
+            any_solid |= v != R(0);
             if constexpr (MOVING) {
                 const int gx = s_gx[cx], gy = s_gyi[cy];
                 R dflt = v, w = R(0), vv = R(0);
-                for (int k = 0; k < A.np; ++k) {
-                    if (!((near >> k) & 1ull)) continue;
+                hits = 0ull;
+                for (unsigned long long m = near; m; m &= m - 1ull) {
+                    const int k = __ffsll((long long)m) - 1;
                     R rx, ry;
                     const R pk = pphi0(k, cx, cy, gx, gy, rx, ry);
+                    if (pk == R(0)) continue;
+                    hits |= 1ull << k;
+                    any_solid = 1;
                     v += pk;
-                    if (A.parts[k].own) {
+                    if ((s_own >> k) & 1ull) {
                         const R ck = s_pv[k][5];
                         w += ck * pk;
                         vv += ck * pk * pk * pk;
@@ -463,9 +474,9 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY, UNIT && 
             racc = rest_own + fix24_to_rest(sold, p.klog2[0]);
         }
         s_phi[ly + 2][lx + 2] = phi_own;
-        const R p0_own = phi0_at(lx + 2, ly + 2);
+        unsigned long long own_hits = 0ull, ring_hits = 0ull;
+        const R p0_own = phi0_at(lx + 2, ly + 2, own_hits);
         s_p0[ly + 2][lx + 2] = p0_own;
-        [[maybe_unused]] int any_solid = p0_own != R(0);
         constexpr int RING = 4 * (TX + 4) + 4 * TY;
         for (int r = tid; r < RING; r += NT) {
             int hx, hy;
@@ -483,9 +494,8 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY, UNIT && 
                 hx = c < 2 ? c : TX + c;
             }
             s_phi[hy][hx] = phi_at(hx, hy, nullptr, nullptr);
-            const R p0 = phi0_at(hx, hy);
+            const R p0 = phi0_at(hx, hy, ring_hits);
             s_p0[hy][hx] = p0;
-            any_solid |= p0 != R(0);
         }
         if constexpr (MODE == MODE_STEP) {
             // w of the own cell from the lagged fields already in registers; the
@@ -523,11 +533,12 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY, UNIT && 
                 }
             }
         }
-        // FP64: a frame without a solid skips the solid's terms of mu_phi, all
-        // zero (a third of stage B's operations)
+        // a frame without a solid skips the solids' terms of mu_phi and of the
+        // force, all zero: in FP64 a third of stage B's operations, with free
+        // particles five stencils
         bool solid_tile = true;
-        if constexpr (UNIT && sizeof(R) == 8)
-            solid_tile = __syncthreads_or(any_solid) || (MOVING && A.wv);
+        if constexpr (MOVING || (UNIT && sizeof(R) == 8))
+            solid_tile = __syncthreads_or(any_solid);
         else
             __syncthreads();
 
@@ -539,7 +550,7 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY, UNIT && 
             const int hx = wx + 1, hy = wy + 1;
             const R ph = s_phi[hy][hx];
             const R lp = lap9<R, FX>(s_phi, hx, hy);
-            if constexpr (UNIT && sizeof(R) == 8) {
+            if constexpr (MOVING || (UNIT && sizeof(R) == 8)) {
                 if (!solid_tile) {
                     s_mu[wy][wx] = c_dw * ph * (ph - R(1)) * (ph + R(1)) - c_lap * lp;
                     continue;
@@ -616,24 +627,26 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY, UNIT && 
         }
         R lphi = R(0);
         if constexpr (MOVING) {
-            // mu_phi0 grad phi0 (Eq. 19) for free particles
-            lphi = lap9<R, FX>(s_phi, hx, hy);
-            R g0x, g0y;
-            grad9<R, FX>(s_p0, hx, hy, g0x, g0y);
-            if (A.wv) {
-                // sum over solids of mu_phi0,s grad phi0_s with their own angles
-                R gWx, gWy, gVx, gVy;
-                grad9<R, WVX>(s_W, hx, hy, gWx, gWy);
-                grad9<R, WVX>(s_V, hx, hy, gVx, gVy);
-                const R pen = c_pen * phi0 * phi * phi;
-                const R aW = c_dw * phi * (phi * phi - R(1)) - c_lap * lphi, aV = c_dw * phi;
-                Fx += pen * g0x + aW * gWx + aV * gVx;
-                Fy += pen * g0y + aW * gWy + aV * gVy;
-            } else {
-                const R mu0 = c_pen * phi0 * phi * phi + c_wet * phi * (R(3) * phi0 * phi0 + phi * phi - R(1)) -
-                              c_wlap * lphi;
-                Fx += mu0 * g0x;
-                Fy += mu0 * g0y;
+            if (solid_tile) {
+                // mu_phi0 grad phi0 (Eq. 19) for free particles
+                lphi = lap9<R, FX>(s_phi, hx, hy);
+                R g0x, g0y;
+                grad9<R, FX>(s_p0, hx, hy, g0x, g0y);
+                if (A.wv) {
+                    // sum over solids of mu_phi0,s grad phi0_s with their own angles
+                    R gWx, gWy, gVx, gVy;
+                    grad9<R, WVX>(s_W, hx, hy, gWx, gWy);
+                    grad9<R, WVX>(s_V, hx, hy, gVx, gVy);
+                    const R pen = c_pen * phi0 * phi * phi;
+                    const R aW = c_dw * phi * (phi * phi - R(1)) - c_lap * lphi, aV = c_dw * phi;
+                    Fx += pen * g0x + aW * gWx + aV * gVx;
+                    Fy += pen * g0y + aW * gWy + aV * gVy;
+                } else {
+                    const R mu0 = c_pen * phi0 * phi * phi + c_wet * phi * (R(3) * phi0 * phi0 + phi * phi - R(1)) -
+                                  c_wlap * lphi;
+                    Fx += mu0 * g0x;
+                    Fy += mu0 * g0y;
+                }
             }
         } else if constexpr (EXT && MODE == MODE_STEP) {
             if (A.mu0) {
@@ -711,16 +724,14 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY, UNIT && 
         // penalty force f = phi0 (u_s - u*) (Sec. 3.2, after Eq. 36)
         R fpx = -phi0 * usx, fpy = -phi0 * usy;
         if constexpr (MOVING) {
-            for (int k = 0; k < A.np; ++k) {
-                if (!((near >> k) & 1ull)) continue;
+            for (unsigned long long m = own_hits; m; m &= m - 1ull) {
+                const int k = __ffsll((long long)m) - 1;
                 R rx, ry;
                 const R pk = pphi0(k, lx + 3, ly + 3, gx, gy, rx, ry);
-                if (pk != R(0)) {
-                    const R usx_k = s_pv[k][2] - s_pv[k][4] * ry;
-                    const R usy_k = s_pv[k][3] + s_pv[k][4] * rx;
-                    fpx += pk * usx_k;
-                    fpy += pk * usy_k;
-                }
+                const R usx_k = s_pv[k][2] - s_pv[k][4] * ry;
+                const R usy_k = s_pv[k][3] + s_pv[k][4] * rx;
+                fpx += pk * usx_k;
+                fpy += pk * usy_k;
             }
         }
         const R ux = usx + R(0.5) * fpx, uy = usy + R(0.5) * fpy;
@@ -933,22 +944,20 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY, UNIT && 
                     __syncthreads();  // s_red and s_redk are free again
                     nj = 0;
                 };
-                for (int k = 0; k < A.np; ++k) {
-                    if (!((near >> k) & 1ull)) continue;
+                for (unsigned long long m = near; m; m &= m - 1ull) {
+                    const int k = __ffsll((long long)m) - 1;
                     R c6[3] = {R(0), R(0), R(0)};
                     bool hit = false;
-                    if (valid) {
+                    if (valid && ((own_hits >> k) & 1ull)) {
+                        hit = true;
                         R rx, ry;
                         const R pk = pphi0(k, lx + 3, ly + 3, gx, gy, rx, ry);
-                        if (pk != R(0)) {
-                            hit = true;
-                            const R usx_k = s_pv[k][2] - s_pv[k][4] * ry;
-                            const R usy_k = s_pv[k][3] + s_pv[k][4] * rx;
-                            const R fx = rho * pk * (usx_k - usx), fy = rho * pk * (usy_k - usy);
-                            c6[0] = -fx;
-                            c6[1] = -fy;
-                            c6[2] = -(rx * fy - ry * fx);
-                        }
+                        const R usx_k = s_pv[k][2] - s_pv[k][4] * ry;
+                        const R usy_k = s_pv[k][3] + s_pv[k][4] * rx;
+                        const R fx = rho * pk * (usx_k - usx), fy = rho * pk * (usy_k - usy);
+                        c6[0] = -fx;
+                        c6[1] = -fy;
+                        c6[2] = -(rx * fy - ry * fx);
                     }
                     const bool wany = __any_sync(0xffffffffu, hit);
 #pragma unroll
