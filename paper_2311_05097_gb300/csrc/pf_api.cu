@@ -511,7 +511,7 @@ struct Engine {
     int2 *d_mtxy = nullptr;
     std::vector<int> mbase, mcount;
     int *d_flags = nullptr;
-    int *d_queue = nullptr;  // work-queue counter of the strip step
+    int *d_queue = nullptr;  // strip step: work-queue counter, and the CTAs that have ended
     double *d_diag = nullptr;  // partials + out
     // particles (single-domain handles)
     ParticleDev hp[PF_MAX_PARTICLES];
@@ -567,6 +567,7 @@ static int engine_setup(Engine &E, int nd, const pf_grid *g, const pf_params *p)
     CK(cudaMalloc(&E.d_flags, sizeof(int) * 4));
     CK(cudaMemset(E.d_flags, 0, sizeof(int) * 4));
     CK(cudaMalloc(&E.d_queue, sizeof(int) * 4));
+    CK(cudaMemset(E.d_queue, 0, sizeof(int) * 4));
     CK(cudaMalloc(&E.d_diag, sizeof(double) * (3 * diag_blocks() + 8)));
     CK(cudaMemset(E.d_diag, 0, sizeof(double) * (3 * diag_blocks() + 8)));
     CK(cudaMalloc(&E.d_parts, sizeof(ParticleDev) * PF_MAX_PARTICLES));
@@ -824,6 +825,7 @@ static StepArgs step_args(const Engine &E, int par)
     a.nitems = E.nitems;
     a.strip_maps = E.d_maps;
     a.dom1 = E.mem.size() == 1 ? &E.mem[0].d : nullptr;
+    a.pdl = E.grid >= E.ntiles && E.ntiles <= 4 * E.nsm;
     return a;
 }
 
@@ -864,10 +866,9 @@ static int issue_step(Engine &E, int par)
     } else if (E.variant == 4) {
         if (!E.ghosts_ok && !launch_any(E, STRIP_SW, 0, MODE_FILL_GHOSTS, (int)E.mem.size(), a))
             return fail(PF_EINVAL, "ghost pass not built");
-        // the items after each CTA's first come from a work queue
+        // the items after each CTA's first come from a work queue (the kernel leaves it at 0)
         StepArgs aq = a;
         aq.queue = E.d_queue;
-        CK(cudaMemsetAsync(E.d_queue, 0, sizeof(int), E.stream));
         if (!launch_any(E, E.tx, E.ty, MODE_STEP_STRIP, E.grid, aq))
             return fail(PF_EINVAL, "strip step of width %d not built", E.tx);
     } else if (!launch_any(E, E.tx, E.ty, step_mode(E), E.grid, a)) {

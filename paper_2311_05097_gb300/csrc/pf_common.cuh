@@ -271,7 +271,9 @@ struct StepArgs {
     int wait_polls;        // polls of one bounded device wait (staged kernel); 0: default
     const unsigned char *tile_sel;  // optional, per tile in device memory: run only the tiles ...
     int sel;                        // ... whose byte equals sel (else every tile)
-    int *queue;            // strip step: work-queue counter (zeroed before the launch), or
+    int pdl;               // single-cell step without particles: one tile per CTA, all resident at once
+                           // (the launch overlaps the step before it)
+    int *queue;            // strip step: work-queue counter (0 at the launch, and left at 0), or
                            // null: static round-robin over the items
     int mu0;               // single-cell step, wall instantiation, no particle terms: the
                            // tiles out of every particle's reach (split step) carry the
@@ -300,6 +302,11 @@ __device__ __forceinline__ __nv_bfloat16 ldg<__nv_bfloat16>(const __nv_bfloat16 
     unsigned short v = __ldg(reinterpret_cast<const unsigned short *>(p));
     return __ushort_as_bfloat16(v);
 }
+
+// a plain load, for kernels that may be resident while their inputs are written
+// (see pdl_begin)
+template <class T>
+__device__ __forceinline__ T ldp(const T *p) { return *p; }
 
 // population store <-> compute conversion
 template <class P>
@@ -488,6 +495,16 @@ __device__ __forceinline__ void bulk_g2s(unsigned dst, const void *src, unsigned
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
                  "l"(src), "r"(bytes), "r"(bar)
                  : "memory");
+}
+// Programmatic dependent launch: waits here until the kernels before this one are
+// complete and their writes visible, then lets the next kernel of the stream be set
+// up while this one runs (it waits here in turn).  Both are no-ops in a kernel
+// launched without the attribute.  A kernel may so be resident while its inputs are
+// written: it reads them with plain loads, not through the read-only path.
+__device__ __forceinline__ void pdl_begin()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 // Wait for the phase of parity `parity` to complete, at most max_iter polls
 // (with back-off); false if it did not.

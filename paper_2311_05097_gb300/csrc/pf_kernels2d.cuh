@@ -265,6 +265,7 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY, UNIT && 
 
     const int tid = threadIdx.x;
     const int lx = tid % TX, ly = tid / TX;
+    if constexpr (MODE == MODE_STEP) pdl_begin();
 
     for (int t = blockIdx.x; t < A.ntiles; t += gridDim.x) {
         if (A.tile_sel && A.tile_sel[t] != A.sel) continue;  // (uniform in the block)
@@ -395,7 +396,7 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY, UNIT && 
                 R movers = R(0);  // sum in stored units, scaled once
 #pragma unroll
                 for (int i = 1; i < 9; ++i) {
-                    ST q = ldg(fs + pull(0, i, cx, cy));
+                    ST q = ldp(fs + pull(0, i, cx, cy));
                     const R v = stored_to_float<ST>(q);
                     if (keep) keep[i] = v * isc1;
                     if (keepq) keepq[i] = q;
@@ -406,7 +407,7 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY, UNIT && 
                 acc = R(0);
 #pragma unroll
                 for (int i = 0; i < 9; ++i) {
-                    R v = Conv<P>::ld(ldg(fs + pull(0, i, cx, cy)), isc1);
+                    R v = Conv<P>::ld(ldp(fs + pull(0, i, cx, cy)), isc1);
                     if (keep) keep[i] = v;
                     acc += v;
                 }
@@ -419,7 +420,7 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY, UNIT && 
         // indicator at this cell is not 0
         auto phi0_at = [&](int hx, int hy, [[maybe_unused]] unsigned long long &hits) -> R {
             const int cx = hx + 1, cy = hy + 1;
-            R v = (R)ldg(ph0 + s_gy[cy] + s_gx[cx]);
+            R v = (R)ldp(ph0 + s_gy[cy] + s_gx[cx]);
             any_solid |= v != R(0);
             if constexpr (MOVING) {
                 const int gx = s_gx[cx], gy = s_gyi[cy];
@@ -456,11 +457,11 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY, UNIT && 
         const int id = s_gy[ly + 3] + s_gx[lx + 3];
         ST f2raw[9];
 #pragma unroll
-        for (int i = 0; i < 9; ++i) f2raw[i] = ldg(fs + pull(9, i, lx + 3, ly + 3));
+        for (int i = 0; i < 9; ++i) f2raw[i] = ldp(fs + pull(9, i, lx + 3, ly + 3));
         AX lag[5];
         if constexpr (MODE == MODE_STEP) {
 #pragma unroll
-            for (int k = 0; k < 5; ++k) lag[k] = ldg(as + k * plane + id);
+            for (int k = 0; k < 5; ++k) lag[k] = ldp(as + k * plane + id);
         }
         R f1[9];
         ST q1[9];
@@ -515,8 +516,8 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY, UNIT && 
                     wx = (rr & 1) ? TX + 1 : 0;
                 }
                 const int wid = s_gy[wy + 2] + s_gx[wx + 2];
-                const R ux = (R)ldg(as + 0 * plane + wid), uy = (R)ldg(as + 1 * plane + wid);
-                const R Sx = (R)ldg(as + 2 * plane + wid), Sy = (R)ldg(as + 3 * plane + wid);
+                const R ux = (R)ldp(as + 0 * plane + wid), uy = (R)ldp(as + 1 * plane + wid);
+                const R Sx = (R)ldp(as + 2 * plane + wid), Sy = (R)ldp(as + 3 * plane + wid);
                 s_w[wy][wx] = wsign(wy + 2) * (Sx * uy - ux * Sy);
             }
         }
@@ -679,8 +680,8 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY, UNIT && 
 #pragma unroll
                 for (int i = -1; i <= 1; ++i) {
                     const int nid = s_gy[ly + 3 + j] + s_gx[lx + 3 + i];
-                    const R ux = (R)ldg(as + 0 * plane + nid), uy = (R)ldg(as + 1 * plane + nid);
-                    const R sx = (R)ldg(as + 2 * plane + nid), sy = (R)ldg(as + 3 * plane + nid);
+                    const R ux = (R)ldp(as + 0 * plane + nid), uy = (R)ldp(as + 1 * plane + nid);
+                    const R sx = (R)ldp(as + 2 * plane + nid), sy = (R)ldp(as + 3 * plane + nid);
                     wv[j + 1][i + 1] = wsign(ly + 3 + j) * (sx * uy - ux * sy);
                 }
             R wgx, wgy;
@@ -741,7 +742,7 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY, UNIT && 
         // macroscopic pass reads them here)
         if constexpr (MODE == MODE_MACROS) {
 #pragma unroll
-            for (int k = 0; k < 5; ++k) lag[k] = ldg(as + k * plane + id);
+            for (int k = 0; k < 5; ++k) lag[k] = ldp(as + k * plane + id);
         }
         const R upx = (R)lag[0], upy = (R)lag[1];
         const R Spx = (R)lag[2], Spy = (R)lag[3];

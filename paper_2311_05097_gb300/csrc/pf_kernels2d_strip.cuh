@@ -239,6 +239,9 @@ __global__ void __launch_bounds__(32 * B, 2) k_step2d_strip(StepArgs A)
         mbar_init(bar(0), 1);
         mbar_init(bar(1), 1);
     }
+    pdl_begin();
+    // (the tensor copies read what the kernel before wrote)
+    asm volatile("fence.proxy.async.global;" ::: "memory");
     unsigned phases = 0u;
     const int polls = A.wait_polls > 0 ? A.wait_polls : STAGE_WAIT_POLLS;
     const char *maps_all = reinterpret_cast<const char *>(A.strip_maps);
@@ -251,6 +254,14 @@ __global__ void __launch_bounds__(32 * B, 2) k_step2d_strip(StepArgs A)
         if (tid == 0) s_next = gridDim.x + atomicAdd(A.queue, 1);
         __syncthreads();
         return s_next;
+    };
+    // the last CTA to end resets the queue for the next step (a memset between the
+    // steps took 1.5 us of each)
+    auto finish = [&]() {
+        if (A.queue && tid == 0) {
+            __threadfence();
+            if (atomicInc(reinterpret_cast<unsigned *>(A.queue) + 1, gridDim.x - 1) == gridDim.x - 1) *A.queue = 0;
+        }
     };
     for (int it = blockIdx.x; it < A.nitems; it = next_item(it)) {
         const int4 item = A.items[it];
@@ -311,6 +322,7 @@ __global__ void __launch_bounds__(32 * B, 2) k_step2d_strip(StepArgs A)
         // wait to land; end the CTA
         auto give_up = [&](int j, bool my_ok) {
             if (tid == 0) atomicOr(A.flags, 4);
+            finish();
             if (!my_ok) mbar_wait_bounded(bar(j & 1), (phases >> (j & 1)) & 1u, STAGE_WAIT_POLLS);
         };
 
@@ -801,6 +813,7 @@ __global__ void __launch_bounds__(32 * B, 2) k_step2d_strip(StepArgs A)
             }
         }
     }
+    finish();
 }
 
 // Refresh the ghost columns of the read buffers (parity par) of every domain:

@@ -632,6 +632,9 @@ __global__ void __launch_bounds__(REP_THREADS) k_particle_repulsion(const Partic
         for (int w = 0; w < REP_THREADS / 32; ++w) v += red[w][tid];
         frep[3 * k + tid] = v;
     }
+    // (ends after the step it runs beside, so that the update, which waits for this
+    // kernel, comes after both; it reads positions, which the step leaves alone)
+    pdl_begin();
 }
 
 // One block per particle; each thread sums a fixed strided set of tiles, then
@@ -646,6 +649,7 @@ __global__ void __launch_bounds__(UPDATE_THREADS) k_particle_update(ParticleDev 
 {
     const int k = blockIdx.x;
     if (k >= np) return;
+    pdl_begin();
     __shared__ double wred[UPDATE_THREADS / 32][6];
     __shared__ double red[1][6];
     double acc[6] = {0, 0, 0, 0, 0, 0};
@@ -701,7 +705,7 @@ __global__ void __launch_bounds__(UPDATE_THREADS) k_particle_update(ParticleDev 
     for (int c = 0; c < 3; ++c) {
         const double Fin = rho_bar * Vp * (pp.u[c] - pp.u_prev[c]);
         const double Tin = If * (pp.w[c] - pp.w_prev[c]);
-        a[c] = (red[0][c] + frep[3 * k + c] + Fin + (1.0 - rho_bar / pp.rho_p) * Mp * p.g[c]) / Mp;
+        a[c] = (red[0][c] + (p.rep_eps > 0.0 ? frep[3 * k + c] : 0.0) + Fin + (1.0 - rho_bar / pp.rho_p) * Mp * p.g[c]) / Mp;
         al[c] = (red[0][3 + c] + Tin) / Ip;
     }
     if (p.dim == 2) {
@@ -794,9 +798,15 @@ void launch_particle_update(ParticleDev *parts, int np, const double *partials, 
                             const DevParams &p, double *frep, int nx, int ny, int nz, int wall_y,
                             const unsigned char *sel, cudaStream_t s)
 {
-    k_particle_repulsion<<<np, REP_THREADS, 0, s>>>(parts, np, p, nx, ny, nz, wall_y, frep);
-    k_particle_update<<<np, UPDATE_THREADS, 0, s>>>(parts, np, partials, ntiles, p, frep, sel);
-    count_launches(2);
+    const bool rep = p.rep_eps > 0.0;
+    if (sel) {  // (the split step: joined from two streams)
+        if (rep) k_particle_repulsion<<<np, REP_THREADS, 0, s>>>(parts, np, p, nx, ny, nz, wall_y, frep);
+        k_particle_update<<<np, UPDATE_THREADS, 0, s>>>(parts, np, partials, ntiles, p, frep, sel);
+    } else {
+        if (rep) launch_pdl(k_particle_repulsion, np, REP_THREADS, 0, s, parts, np, p, nx, ny, nz, wall_y, frep);
+        launch_pdl(k_particle_update, np, UPDATE_THREADS, 0, s, parts, np, partials, ntiles, p, frep, sel);
+    }
+    count_launches(rep ? 2 : 1);
 }
 
 }  // namespace pf
