@@ -90,7 +90,7 @@ __device__ __forceinline__ void collide9_unit_phi(R f[9], R phi, R j1, R j2, R c
     const R a = ku.h1c * cs2_eta_mu, b1 = ku.h1c * j1, b2 = ku.h1c * j2;  // (1 - cs2)/2
     const R q8 = ku.qc * cs2_eta_mu, c1 = ku.qc * j1, c2 = ku.qc * j2;    // cs2/4
     const R s = c1 + c2, d = c1 - c2;
-    f[0] = phi - R(2) * cs2_eta_mu + ku.cs2 * cs2_eta_mu;
+    f[0] = phi - R(2) * cs2_eta_mu + ku.c * cs2_eta_mu;
     f[1] = a + b1;
     f[3] = a - b1;
     f[2] = a + b2;
