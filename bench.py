@@ -692,9 +692,9 @@ def run_single_large(args, dist, rank, world, local, case, prec, cells, bpc, sim
                 clk=clk, launches=launches, e2e=e2e, t_wall=t_wall, kernel=kernel)
 
 
-# FP64 instructions per 2D cell update of the FP64 step (DADD + DMUL + DFMA thread
-# instructions per cell from ncu on the batched workload, kernel 0)
-FP64_INST_PER_CELL_2D = 422.1
+# FP64 instructions per 2D cell update of the FP64 step at unit rates (DADD + DMUL +
+# DFMA thread instructions per cell from ncu on a batch of drops on a wall, kernel 0)
+FP64_INST_PER_CELL_2D = 275.1
 GB300_SMS = 152
 FP64_INST_PER_CLK_PER_SM = 2  # DFMA/DADD/DMUL issue rate of one SM (ncu peak_sustained)
 

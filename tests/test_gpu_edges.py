@@ -214,3 +214,21 @@ def test_tuned_strip_segments(pf, shapes):
         x, y = b.macros(i), s.macros()
         # FP32 roundings of 256 steps (random: 6e-8 sqrt(256) of phi, 16 times that as the fields' bound)
         assert np.abs(x["phi"] - y["phi"]).max() <= 2e-5, i
+
+
+@pytest.mark.parametrize("d0", [0.4, 0.3, 1.0 / 3.0])
+def test_unit_rates_keep_momentum_fp32(pf, d0):
+    """A uniform flow without an interface keeps its velocity: the FP32 step's weights of a moment's axis and
+    diagonal shares add up exactly, so only roundings remain (6e-8 a step, as a random walk over 200 steps; a
+    drift of 3e-8 a step would reach 6e-6)."""
+    c = W.small_case((20, 36), seed=1, solid=False, rho_ratio=1.0, mu_ratio=1.0)
+    c["params"].update(d0=d0, s0=1.6)
+    u = np.zeros((2, 20, 36))
+    u[0], u[1] = 0.013, -0.007
+    g = pf.Sim(c["shape"], precision="p32", **c["params"])
+    g.init(c["phi0"], np.ones(c["shape"]), u)
+    g.set_config(32, 8, 0, 0)
+    g.step(200)
+    m = g.macros()
+    for a in range(2):
+        assert abs(m["u"][a].mean() / u[a, 0, 0] - 1.0) <= 6e-8 * np.sqrt(200.0) * 2.0
