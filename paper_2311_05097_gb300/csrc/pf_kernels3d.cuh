@@ -293,13 +293,17 @@ __device__ __forceinline__ const DomainDev &tile_of(const StepArgs &A, const Dom
 // the plane of phi of the step under way (k_phi3d)
 __device__ __forceinline__ float *phi_of_step(const DomainDev &Dm) { return reinterpret_cast<float *>(Dm.phi0) + Dm.plane; }
 
-// One particle near a tile, in the arithmetic type: the image nearest to the
-// tile as whole cells (ix, iy, iz, in the tile's coordinates) and a fraction,
-// so that a cell's offset R(cell - i) - f is rounded once, as (R) of the FP64
-// difference is.
+// One particle near a tile, in the arithmetic type: its centre as whole cells
+// (ix, iy, iz) and a fraction, so that a cell's offset R(cell - i) - f is rounded
+// once, as (R) of the FP64 difference is.  fast: the whole cells are those of the
+// image nearest to the tile, in the tile's coordinates, and serve every cell of
+// its frames.  Otherwise (the box is too small for one image, or the frames hold
+// mirror rows) they are the domain's, 0 .. n - 1, and each cell takes its minimum
+// image from its own wrapped coordinates: a table coordinate may lie several
+// lengths of a box narrower than the tile from the image.
 template <class R>
 struct Near3 {
-    int ix, iy, iz, k, own, fast;  // fast 0: the box is too small for one image (or mirror rows), wrapped per cell
+    int ix, iy, iz, k, own, fast;
     R fx, fy, fz, Rp, lim2, ct;
     R u[3], w[3];
 };
@@ -459,9 +463,9 @@ __global__ void __launch_bounds__(TX *TY, (sizeof(typename P::real) == 4 && !MOV
                         }
                         hit = e2 < (reach + 1.0) * (reach + 1.0);
                         const double fl[3] = {floor(c[0]), floor(c[1]), floor(c[2])};
-                        q.ix = (int)fl[0] - x0;
-                        q.iy = (int)fl[1] - y0;
-                        q.iz = (int)fl[2] - z0;
+                        q.ix = fast ? (int)fl[0] - x0 : wrap_idx((int)fl[0], nx);
+                        q.iy = fast ? (int)fl[1] - y0 : (wall ? (int)fl[1] : wrap_idx((int)fl[1], ny));
+                        q.iz = fast ? (int)fl[2] - z0 : wrap_idx((int)fl[2], nz);
                         q.fx = (R)(c[0] - fl[0]);
                         q.fy = (R)(c[1] - fl[1]);
                         q.fz = (R)(c[2] - fl[2]);
@@ -487,39 +491,33 @@ __global__ void __launch_bounds__(TX *TY, (sizeof(typename P::real) == 4 && !MOV
             __syncthreads();
         }
         [[maybe_unused]] const int nn = MOVING ? s_nn : 0;
-        // component of a cell's offset to a particle: its minimum image (min_image's
-        // rule, without FP64: the whole cells are wrapped before the one rounding)
+        // component of a cell's offset to a particle, both in the domain: its minimum
+        // image (min_image's rule, without FP64: |d| < n, so one shift of the whole
+        // cells reaches it, before the one rounding)
         [[maybe_unused]] auto wrapped = [](int d, R f, int n) -> R {
-            R r = R(d) - f;
-            const R half = R(0.5) * R(n);
-            if (r > half) r = R(d - n) - f;
-            else if (r < -half) r = R(d + n) - f;
+            const R r = R(d) - f, half = R(0.5) * R(n);
+            if (r > half) return R(d - n) - f;
+            if (r < -half) return R(d + n) - f;
             return r;
         };
         // offset of cell (table cx, cy of the tile + 3 frame; plane z of the chunk's
         // run z0 - 2 ..) to near particle q, and its indicator there
         [[maybe_unused]] auto near_at = [&](const Near3<R> &q, int cx, int cy, int z, R &rx, R &ry, R &rz) -> R {
-            const int dx = cx - 3 - q.ix, dz = z - z0 - q.iz;
-            int dy = cy - 3 - q.iy;
             if (q.fast) {
-                rx = R(dx) - q.fx;
-                ry = R(dy) - q.fy;
-                rz = R(dz) - q.fz;
+                rx = R(cx - 3 - q.ix) - q.fx;
+                ry = R(cy - 3 - q.iy) - q.fy;
+                rz = R(z - z0 - q.iz) - q.fz;
             } else {
-                rx = wrapped(dx, q.fx, nx);
-                rz = wrapped(dz, q.fz, nz);
-                if (EXT && wall) {
-                    dy = s_gyi[cy] - y0 - q.iy;  // (mirror rows; no image across a wall)
-                    ry = R(dy) - q.fy;
-                } else {
-                    ry = wrapped(dy, q.fy, ny);
-                }
+                rx = wrapped(s_gx[cx] - q.ix, q.fx, nx);
+                const int dy = s_gyi[cy] - q.iy;  // (no image across a wall)
+                ry = EXT && wall ? R(dy) - q.fy : wrapped(dy, q.fy, ny);
+                rz = wrapped(wrap_near(z, nz) - q.iz, q.fz, nz);
             }
             return near_phi0_3d<R>(q, rx, ry, rz, (R)p.D);
         };
         // whether near particle q may reach plane z (uniform)
         [[maybe_unused]] auto meets = [&](const Near3<R> &q, int z) -> bool {
-            const R dz = wrapped(z - z0 - q.iz, q.fz, nz);
+            const R dz = q.fast ? R(z - z0 - q.iz) - q.fz : wrapped(wrap_near(z, nz) - q.iz, q.fz, nz);
             return dz * dz < q.lim2;
         };
         // a tile whose frames reach beyond a wall

@@ -232,3 +232,36 @@ def test_unit_rates_keep_momentum_fp32(pf, d0):
     m = g.macros()
     for a in range(2):
         assert abs(m["u"][a].mean() / u[a, 0, 0] - 1.0) <= 6e-8 * np.sqrt(200.0) * 2.0
+
+
+# boxes narrower than the tile (32 x 8 in FP32 arithmetic, 16 x 8 in FP64) in x and y, down to the smallest:
+# frame cells lie several box lengths from a particle's nearest image
+@pytest.mark.parametrize("precision,shape,walls", [
+    ("p32", (9, 7, 4), False), ("p32", (5, 4, 8), False), ("p32", (7, 9, 11), True), ("p32", (10, 5, 16), False),
+    ("p32", (4, 6, 17), True), ("fp16", (8, 5, 6), False), ("fp16", (6, 9, 15), True),
+    ("p64", (8, 9, 5), False), ("p64", (4, 5, 6), False), ("p64", (9, 4, 9), False), ("p64", (6, 7, 7), True),
+    ("p64", (4, 4, 4), False),
+])
+def test_moving_3d_narrow_boxes(pf, precision, shape, walls):
+    """The minimum image of the 3D particle step in boxes of less than a tile: FP64 at 1e-12; FP32 and the
+    16-bit policy within a few roundings of four steps (6e-8; movers 2^-11 of sizes below 0.02)."""
+    nz, ny, nx = shape
+    c = W.small_case(shape, seed=9, solid=False, u_amp=0.005, rho_ratio=1.0, mu_ratio=1.0, D=2.0)
+    c["params"].update(solid_eps=0.1)
+    R = min(2.0, 0.25 * min(shape))
+    # (no cell exactly half a box from a centre: its minimum image is not unique)
+    parts = [dict(x=(0.46 * nx + 0.03, 0.5 * ny + 0.31, 0.6 * nz + 0.07), u=(0.01, 0.002, -0.004), w=(0.001, 0.0, 0.002),
+                  R=R, rho_p=2.0),
+             dict(x=(0.9 * nx + 0.01, 0.3 * ny + 0.11, nz - 0.7), u=(0.0, 0.01, 0.0), R=0.8 * R, rho_p=1.5, theta_deg=60.0)]
+    for q in parts:
+        c["phi"] = (1.0 - W.disc(shape, q["x"], q["R"], 2.0)) * c["phi"]
+    g, o = _pair(pf, c, 4, precision=precision, particles=parts, walls=walls)
+    gm, om = g.macros(), o.macros()
+    tol = dict(p64=(1e-12, 1e-12, 1e-12), p32=(2e-6, 1e-4, 1e-4), fp16=(1e-4, 2e-2, 2e-2))[precision]
+    for k, t in zip(("phi", "u", "P"), tol):
+        assert np.abs(gm[k] - om[k]).max() <= t * max(np.abs(om[k]).max(), 1e-3), k
+    F = max(np.abs(np.array(o.particle(k).F)).max() for k in range(2))
+    for k in range(2):
+        pg, po = g.particle(k), o.particle(k)
+        assert np.abs(np.array(pg["x"]) - np.array(po.x)).max() <= 1e-6 * max(shape), k
+        assert np.abs(np.array(pg["F"]) - np.array(po.F)).max() <= (1e-11 if precision == "p64" else 2e-3) * F, k
