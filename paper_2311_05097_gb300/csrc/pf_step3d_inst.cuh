@@ -1,6 +1,7 @@
 // Instantiation and dispatch of the 3D step kernel for one precision policy.
 #pragma once
 
+#include "pf.h"
 #include "pf_internal.h"
 #include "pf_kernels3d_pair.cuh"
 
@@ -12,7 +13,10 @@ static bool run3d(int grid, cudaStream_t s, const StepArgs &a, int *occ)
     using R = typename P::real;
     auto kern = k_step3d<P, TX, TY, MOVING, MODE, EXT, UNIT>;
     const int dyn = MOVING ? (int)step3d_moving_smem<R, TX, TY>(a.np, a.wv) : 0;
-    if (dyn && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn) != cudaSuccess)
+    // the limit is the function's, shared by every simulation and host thread: always
+    // the largest size, so that no launch finds it below its own
+    constexpr int dyn_max = MOVING ? (int)step3d_moving_smem<R, TX, TY>(PF_MAX_PARTICLES, true) : 0;
+    if (dyn && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn_max) != cudaSuccess)
         return false;
     if (occ) {
         int n = 0;

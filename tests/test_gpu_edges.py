@@ -265,3 +265,34 @@ def test_moving_3d_narrow_boxes(pf, precision, shape, walls):
         pg, po = g.particle(k), o.particle(k)
         assert np.abs(np.array(pg["x"]) - np.array(po.x)).max() <= 1e-6 * max(shape), k
         assert np.abs(np.array(pg["F"]) - np.array(po.F)).max() <= (1e-11 if precision == "p64" else 2e-3) * F, k
+
+
+def test_moving_3d_simulations_on_several_threads(pf):
+    """Host threads launch the same 3D kernels with different numbers of particles: the dynamic shared memory that
+    the larger ones need stays allowed whatever the others launch in between."""
+    import threading
+
+    def sim(count):
+        c = W.small_case((12, 14, 40), seed=2, solid=False)
+        s = pf.Sim(c["shape"], precision="p32", **c["params"])
+        for k in range(count):
+            s.set_particle(k, x=(4.0 + 0.65 * k, 5.0 + 0.1 * k, 6.0), R=1.5, rho_p=1.5, theta_deg=60.0)
+        s.init(c["phi0"], c["phi"])
+        s.step(2)
+        return s
+
+    failed = []
+
+    def work(s, n):
+        try:
+            for _ in range(n):
+                s.diagnostics()
+        except pf.PfError as e:
+            failed.append(str(e))
+
+    threads = [threading.Thread(target=work, args=(sim(count), 4000)) for count in (1, 1, 1, 50, 50)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failed, failed
