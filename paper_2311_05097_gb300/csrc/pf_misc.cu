@@ -553,6 +553,9 @@ __global__ void __launch_bounds__(REP_THREADS) k_particle_repulsion(const Partic
 {
     const int k = blockIdx.x, tid = threadIdx.x;
     if (k >= np) return;
+    // (before the first read: the positions are the update's of the step before, and only
+    // this kernel's own wait makes them visible to it)
+    pdl_begin();
     __shared__ double red[REP_THREADS / 32][3];
     double acc[3] = {0.0, 0.0, 0.0};
     if (p.rep_eps > 0.0) {
@@ -632,9 +635,6 @@ __global__ void __launch_bounds__(REP_THREADS) k_particle_repulsion(const Partic
         for (int w = 0; w < REP_THREADS / 32; ++w) v += red[w][tid];
         frep[3 * k + tid] = v;
     }
-    // (ends after the step it runs beside, so that the update, which waits for this
-    // kernel, comes after both; it reads positions, which the step leaves alone)
-    pdl_begin();
 }
 
 // One block per particle; each thread sums a fixed strided set of tiles, then

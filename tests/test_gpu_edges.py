@@ -296,3 +296,35 @@ def test_moving_3d_simulations_on_several_threads(pf):
     for t in threads:
         t.join()
     assert not failed, failed
+
+
+@pytest.mark.parametrize("shape,count", [((64, 72), 12), ((40, 40, 44), 6)])
+@pytest.mark.parametrize("precision", ["p64", "fp16"])
+def test_repulsion_in_one_call_equals_single_steps(pf, shape, count, precision):
+    """Particles that push one another, every step's launches following on at once (one call of many steps) and
+    each step waited for: the same bits."""
+    c = W.small_case(shape, seed=3, solid=False, rho_ratio=1.0, mu_ratio=1.0)
+    c["params"].update(rep_xi=2.5, rep_eps=1e4, solid_eps=0.1)
+    n = list(reversed(shape))
+    parts = []
+    for k in range(count):
+        i = np.array([k % 3, k // 3 % 4, k % 2])[:len(n)]
+        parts.append(dict(x=[float(v) for v in 14.2 * i + 9.1], u=[0.002 * (-1) ** k] + [0.0] * (len(n) - 1), R=6.0, rho_p=3.0))
+        c["phi"] = (1.0 - W.disc(shape, parts[-1]["x"], 6.0, 4.0)) * c["phi"]
+    sims = []
+    for _ in range(2):
+        s = pf.Sim(shape, precision=precision, **c["params"])
+        for k, q in enumerate(parts):
+            s.set_particle(k, **q)
+        s.init(c["phi0"], c["phi"])
+        s.set_config(16 if len(n) == 3 and precision == "p64" else 32, 8, 0, 0)
+        sims.append(s)
+    sims[0].step(48)
+    for _ in range(48):
+        sims[1].step(1)
+        sims[1].sync()
+    for k in range(count):
+        a, b = sims[0].particle(k), sims[1].particle(k)
+        assert all(a[f] == b[f] for f in ("x", "u", "w", "F", "T")), k
+        assert a["x"][0] != parts[k]["x"][0]
+    assert np.array_equal(sims[0].macros()["phi"], sims[1].macros()["phi"])
