@@ -206,7 +206,8 @@ int pf_autotune(pf_handle *h, int64_t *steps_taken);
 
 /* Macroscopic fields at the current time recomputed from the populations
  * (Eqs. 31, 17, 36): phi (N), rho (N), u (dim*N), P (N), mu = mu_phi of Eq. (9)
- * (N).  NULL outputs are skipped.  Synchronous. */
+ * (N).  NULL outputs are skipped.  Synchronous.  After a step that timed out
+ * (PF_ETIMEOUT) the outputs are left as they were. */
 int pf_get_macros(pf_handle *h, double *phi, double *rho, double *u, double *P, double *mu,
                   int where);
 

@@ -1538,33 +1538,6 @@ static MacroOut wanted(const Engine &E, int i, double *phi, double *rho, double 
     return {phi, rho, u, P, mu, nullptr, nullptr, nullptr};
 }
 
-// the macroscopic pass of domain i and the copies of the requested fields,
-// queued on the engine's stream (the caller waits)
-static int engine_queue_macros(Engine &E, int i, double *phi, double *rho, double *u, double *P, double *mu,
-                               int where)
-{
-    if (where == PF_DEVICE) {
-        // written by the pass itself: no buffer, no copies (512^2: 54 us a call with them)
-        std::vector<OutRange> r;
-        const MacroOut out = wanted(E, i, phi, rho, u, P, mu, r);
-        if (direct_outputs(r)) return engine_macros_to(E, i, out);
-    }
-    int rc = engine_macros(E, i);
-    if (rc) return rc;
-    const DomainMem &m = E.mem[i];
-    const long long N = (long long)m.d.nx * m.d.ny * m.d.nz;
-    const cudaMemcpyKind kind = where == PF_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
-    const int d = E.dim;
-    const double *mac = E.d_macro;
-    // stream-ordered copies after the macroscopic pass, then one wait
-    if (phi) CK(cudaMemcpyAsync(phi, mac, sizeof(double) * N, kind, E.stream));
-    if (rho) CK(cudaMemcpyAsync(rho, mac + N, sizeof(double) * N, kind, E.stream));
-    if (u) CK(cudaMemcpyAsync(u, mac + 2 * N, sizeof(double) * d * N, kind, E.stream));
-    if (P) CK(cudaMemcpyAsync(P, mac + (2 + d) * N, sizeof(double) * N, kind, E.stream));
-    if (mu) CK(cudaMemcpyAsync(mu, mac + (3 + d) * N, sizeof(double) * N, kind, E.stream));
-    return PF_OK;
-}
-
 static int engine_get_macros(Engine &E, int i, double *phi, double *rho, double *u, double *P,
                              double *mu, int where)
 {
@@ -1572,8 +1545,18 @@ static int engine_get_macros(Engine &E, int i, double *phi, double *rho, double 
     if (where != PF_HOST && where != PF_DEVICE) return fail(PF_EINVAL, "where must be PF_HOST or PF_DEVICE");
     if (!E.inited[i]) return fail(PF_ESTATE, "pf_get_macros before pf_init_fields");
     if (E.sticky) return E.sticky;
-    // queued behind the steps, one wait: the steps' flags come with it
-    int rc = engine_queue_macros(E, i, phi, rho, u, P, mu, where);
+    // the pass is queued behind the steps and their flags come with it.  Device arrays
+    // are written by the pass itself (no buffer, no copies: 512^2: 54 us a call with
+    // them), which leaves them alone after a step that timed out; other arrays are
+    // copied to once the flags are known
+    bool direct = false;
+    MacroOut out{};
+    if (where == PF_DEVICE) {
+        std::vector<OutRange> r;
+        out = wanted(E, i, phi, rho, u, P, mu, r);
+        direct = direct_outputs(r);
+    }
+    int rc = direct ? engine_macros_to(E, i, out) : engine_macros(E, i);
     int flag = 0;
     const cudaError_t ce = cudaMemcpyAsync(&flag, E.d_flags, sizeof(int), cudaMemcpyDeviceToHost, E.stream);
     const int wrc = engine_wait(E);
@@ -1581,7 +1564,20 @@ static int engine_get_macros(Engine &E, int i, double *phi, double *rho, double 
     if (rc) return rc;
     CK(ce);
     rc = flags_rc(E, flag);
-    return rc == PF_ENUMERIC ? PF_OK : rc;
+    if (rc && rc != PF_ENUMERIC) return rc;
+    if (direct) return PF_OK;
+    const DomainMem &m = E.mem[i];
+    const long long N = (long long)m.d.nx * m.d.ny * m.d.nz;
+    const cudaMemcpyKind kind = where == PF_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
+    const int d = E.dim;
+    const double *mac = E.d_macro;
+    if (phi) CK(cudaMemcpyAsync(phi, mac, sizeof(double) * N, kind, E.stream));
+    if (rho) CK(cudaMemcpyAsync(rho, mac + N, sizeof(double) * N, kind, E.stream));
+    if (u) CK(cudaMemcpyAsync(u, mac + 2 * N, sizeof(double) * d * N, kind, E.stream));
+    if (P) CK(cudaMemcpyAsync(P, mac + (2 + d) * N, sizeof(double) * N, kind, E.stream));
+    if (mu) CK(cudaMemcpyAsync(mu, mac + (3 + d) * N, sizeof(double) * N, kind, E.stream));
+    CK(cudaStreamSynchronize(E.stream));
+    return PF_OK;
 }
 
 // interface normal n = grad phi / |grad phi| of domain i (0 where |grad phi|^2 <= 1e-24)

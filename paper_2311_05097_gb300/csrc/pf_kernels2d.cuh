@@ -265,6 +265,9 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY, UNIT && 
 
     const int tid = threadIdx.x;
     const int lx = tid % TX, ly = tid / TX;
+    // a step that timed out (bit 2) leaves no fields to read: nothing is written
+    [[maybe_unused]] int lost = 0;
+    if constexpr (MODE == MODE_MACROS) lost = *A.flags & 4;
     if constexpr (MODE == MODE_STEP) pdl_begin();
 
     for (int t = blockIdx.x; t < A.ntiles; t += gridDim.x) {
@@ -772,7 +775,7 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY, UNIT && 
                                  Kf * R(0.5) * dt_term);
 
         if constexpr (MODE == MODE_MACROS) {
-            if (valid) {
+            if (valid && !lost) {
                 const long long N = (long long)nx * ny;
                 const long long o = (long long)gy * nx + gx;
                 double phv = (double)phi;

@@ -392,6 +392,9 @@ __global__ void __launch_bounds__(TX *TY, (sizeof(typename P::real) == 4 && !MOV
 
     const int tid = threadIdx.x;
     const int lx = tid % TX, ly = tid / TX;
+    // a step that timed out (bit 2) leaves no fields to read: nothing is written
+    [[maybe_unused]] int lost = 0;
+    if constexpr (MODE == MODE_MACROS) lost = *A.flags & 4;
 
     for (int t = blockIdx.x; t < A.ntiles; t += gridDim.x) {
         int tx, ty, tz;
@@ -921,7 +924,7 @@ __global__ void __launch_bounds__(TX *TY, (sizeof(typename P::real) == 4 && !MOV
                                       Kf * R(0.5) * dt_term);
 
             if constexpr (MODE == MODE_MACROS) {
-                if (valid) {
+                if (valid && !lost) {
                     const long long N = (long long)nx * ny * nz;
                     const long long o = ((long long)z * ny + gy) * nx + gx;
                     double phv = (double)phi;

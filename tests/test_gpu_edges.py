@@ -328,3 +328,41 @@ def test_repulsion_in_one_call_equals_single_steps(pf, shape, count, precision):
         assert all(a[f] == b[f] for f in ("x", "u", "w", "F", "T")), k
         assert a["x"][0] != parts[k]["x"][0]
     assert np.array_equal(sims[0].macros()["phi"], sims[1].macros()["phi"])
+
+
+@pytest.mark.parametrize("where", ["direct", "overlapping", "host"])
+def test_timed_out_step_leaves_outputs_alone(pf, monkeypatch, where):
+    """A readback after a step whose bounded wait ran out returns the error and writes nothing into the caller's
+    arrays: those the pass writes itself, those it copies to, one domain and a whole batch."""
+    import ctypes as C
+    import torch
+    shapes = [(32, 64), (40, 96)]
+    cases = [W.small_case(s, seed=1, solid=False) for s in shapes]
+    for batch in (False, True):
+        monkeypatch.setenv("PF_WAIT_POLLS", "1")
+        if batch:
+            g = pf.Batch(shapes, [c["params"] for c in cases], precision="fp16")
+        else:
+            g = pf.Sim(shapes[0], precision="fp16", **cases[0]["params"])
+        monkeypatch.delenv("PF_WAIT_POLLS")
+        if batch:
+            g.init_all([c["phi0"] for c in cases], [c["phi"] for c in cases])
+        else:
+            g.init(cases[0]["phi0"], cases[0]["phi"])
+        g.set_config(64, 128, 4)
+        g.step(1)
+        bufs = [torch.full((6 * s[0] * s[1],), 7.0, dtype=torch.float64, device="cpu" if where == "host" else "cuda")
+                for s in shapes]
+        N = [s[0] * s[1] for s in shapes]
+        ptrs = []
+        for k in range(5):  # phi, rho, u, P, mu (overlapping: rho over phi)
+            at = {"overlapping": [0, 0, 2, 4, 5]}.get(where, [0, 1, 2, 4, 5])[k]
+            ptrs.append([b.data_ptr() + 8 * at * n for b, n in zip(bufs, N)])
+        w = pf.PF_HOST if where == "host" else pf.PF_DEVICE
+        if batch:
+            tables = [C.cast((C.c_void_p * 2)(*p), C.c_void_p) for p in ptrs]
+            rc = pf.load().pf_batch_get_macros_all(g._h, *tables, w)
+        else:
+            rc = pf.load().pf_get_macros(g._h, *[C.c_void_p(p[0]) for p in ptrs], w)
+        assert rc == pf.PF_ETIMEOUT
+        assert all(bool((b == 7.0).all()) for b in bufs)
