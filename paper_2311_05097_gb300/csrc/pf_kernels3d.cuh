@@ -293,26 +293,66 @@ __device__ __forceinline__ const DomainDev &tile_of(const StepArgs &A, const Dom
 // the plane of phi of the step under way (k_phi3d)
 __device__ __forceinline__ float *phi_of_step(const DomainDev &Dm) { return reinterpret_cast<float *>(Dm.phi0) + Dm.plane; }
 
-// One particle near a tile, in the arithmetic type: its centre as whole cells
-// (ix, iy, iz) and a fraction, so that a cell's offset R(cell - i) - f is rounded
-// once, as (R) of the FP64 difference is.  fast: the whole cells are those of the
-// image nearest to the tile, in the tile's coordinates, and serve every cell of
-// its frames.  Otherwise (the box is too small for one image, or the frames hold
-// mirror rows) they are the domain's, 0 .. n - 1, and each cell takes its minimum
-// image from its own wrapped coordinates: a table coordinate may lie several
-// lengths of a box narrower than the tile from the image.
+// One particle near a tile: its centre as whole cells i and a fraction in two
+// parts of the arithmetic type (fh + fl: FP64 holds it in fh alone, two FP32
+// parts to 48 bits).  fast: the whole cells are those of the image nearest to the
+// tile, in the tile's coordinates, and serve every cell of its frames.  Otherwise
+// (the box is too small for one image, or the frames hold mirror rows) they are
+// the domain's, 0 .. n - 1, and each cell takes its minimum image from its own
+// wrapped coordinates: a table coordinate may lie several lengths of a box
+// narrower than the tile from the image.
 template <class R>
 struct Near3 {
-    int ix, iy, iz, k, own, fast;
-    R fx, fy, fz, Rp, lim2, ct;
+    int i[3], k, own, fast;
+    R fh[3], fl[3], Rp, lim2, ct;
     R u[3], w[3];
 };
 
+// A component of a cell's offset, d - f for whole cells d: h is the difference
+// rounded once, h + l the difference (FP32: to 2^-48; FP64: l = 0).
 template <class R>
-__device__ __forceinline__ R near_phi0_3d(const Near3<R> &q, R rx, R ry, R rz, R D)
+struct Off {
+    R h, l;
+};
+template <class R>
+__device__ __forceinline__ Off<R> near_off(int d, R fh, R fl)
 {
-    const R r2 = rx * rx + ry * ry + rz * rz;
+    const R a = R(d), s = a - fh;
+    if constexpr (sizeof(R) == 8) return {s, R(0)};
+    const R e = ((a - s) - fh) - fl;  // (a - s) - fh is exact: |a| >= fh or a = 0
+    const R h = s + e;
+    return {h, e - (h - s)};
+}
+
+// Indicator at an offset.  FP32: the squares and their sum carry their rounding
+// errors (two-term products and sums), so the squared distance is rounded once, as
+// that of FP64 arithmetic is, whose pipe (two lanes per SM and clock) stays free.
+// Three placements of three spheres in 96 x 80 x 112: 194, 209 and 232 us per step;
+// with plain FP32 sums, an ulp of R off in the distance, 189, 211 and 227.
+template <class R>
+__device__ __forceinline__ R near_phi0_3d(const Near3<R> &q, Off<R> x, Off<R> y, Off<R> z, R D)
+{
+    // (FP32: the indicator is 0 well inside this sum's roundings of the limit, so it
+    // decides the reach)
+    R r2 = x.h * x.h + y.h * y.h + z.h * z.h;
     if (r2 >= q.lim2) return R(0);
+    if constexpr (sizeof(R) == 4) {
+        auto square = [](Off<R> o, R &err) -> R {
+            const R p = __fmul_rn(o.h, o.h);
+            err = __fmaf_rn(o.h + o.h, o.l, __fmaf_rn(o.h, o.h, -p));
+            return p;
+        };
+        auto add = [](R a, R b, R &err) -> R {
+            const R s = a + b, t = s - a;
+            err += (a - (s - t)) + (b - t);
+            return s;
+        };
+        R ex, ey, ez;
+        const R px = square(x, ex), py = square(y, ey), pz = square(z, ez);
+        R err = (ex + ey) + ez;
+        const R s = add(add(px, py, err), pz, err);
+        r2 = s + err;
+    }
     return R(0.5) * (R(1) + tanh(R(2) * (q.Rp - sqrt(r2)) / D));
 }
 
@@ -356,8 +396,9 @@ constexpr size_t step3d_moving_smem(int np, bool wv)
 // (one barrier per chunk; before, every cell of every frame evaluated every
 // particle in FP64 and a barrier followed each particle and plane: 4055 thread
 // instructions per cell, one block of 202 registers per SM).  Three spheres in
-// 96 x 80 x 112 (FP32): 1240 us per step, 925 with the shorter chunks, 177 now;
-// with the FP64 minimum image per cell kept for boxes below 2 reach + tile, 501.  In FP32
+// 96 x 80 x 112 (FP32): 1240 us per step, 925 with the shorter chunks, 190 to 230 by
+// their places now; with the FP64 minimum image per cell kept for boxes below 2 reach
+// + tile, 501.  In FP32
 // arithmetic phi comes from k_phi3d's plane, as in k_step3d_pair, and the
 // domain's descriptor is a kernel parameter.
 template <class P, int TX, int TY, bool MOVING, int MODE, bool EXT, bool UNIT = false>
@@ -450,33 +491,36 @@ __global__ void __launch_bounds__(TX *TY, (sizeof(typename P::real) == 4 && !MOV
                         const double ext[3] = {0.5 * TX + 2.0, 0.5 * TY + 2.0, 0.5 * zc + 2.0};
                         const int n3[3] = {nx, ny, nz}, len[3] = {TX, TY, zc};
                         const double reach = pp.R + indicator_cut<R>(p);
-                        double c[3], e2 = 0.0;
+                        double e2 = 0.0, cell[3];
                         bool fast = true;
 #pragma unroll
                         for (int a = 0; a < 3; ++a) {
                             double dd = mid[a] - pp.x[a];
                             const bool bounded = a == 1 && wall;
-                            if (!bounded) dd = min_image(dd, n3[a]);
-                            c[a] = mid[a] - dd;  // the image nearest to the tile
+                            // the image nearest to the tile is `shift` box lengths away
+                            const double shift = bounded ? 0.0 : n3[a] * rint(dd / n3[a]);
+                            dd -= shift;
                             const double ex = fmax(fabs(dd) - ext[a], 0.0);
                             e2 += ex * ex;
+                            const double whole = floor(pp.x[a]), frac = pp.x[a] - whole;
+                            cell[a] = whole + shift;
+                            q.fh[a] = (R)frac;
+                            q.fl[a] = (R)(frac - (double)q.fh[a]);
                             // with walls rows beyond them are mirror rows: their cells are not
                             // where the table says
                             fast = fast && (bounded ? !(y0 - 3 < 0 || y0 + TY + 3 > ny) : n3[a] >= 2.0 * reach + 6.0 + len[a]);
                         }
                         hit = e2 < (reach + 1.0) * (reach + 1.0);
-                        const double fl[3] = {floor(c[0]), floor(c[1]), floor(c[2])};
-                        q.ix = fast ? (int)fl[0] - x0 : wrap_idx((int)fl[0], nx);
-                        q.iy = fast ? (int)fl[1] - y0 : (wall ? (int)fl[1] : wrap_idx((int)fl[1], ny));
-                        q.iz = fast ? (int)fl[2] - z0 : wrap_idx((int)fl[2], nz);
-                        q.fx = (R)(c[0] - fl[0]);
-                        q.fy = (R)(c[1] - fl[1]);
-                        q.fz = (R)(c[2] - fl[2]);
+                        const int at[3] = {x0, y0, z0};
+#pragma unroll
+                        for (int a = 0; a < 3; ++a)
+                            q.i[a] = fast ? (int)cell[a] - at[a]
+                                          : (a == 1 && wall ? (int)cell[a] : wrap_idx((int)cell[a], n3[a]));
                         q.k = k;
                         q.own = pp.own;
                         q.fast = fast;
                         q.Rp = (R)pp.R;
-                        q.lim2 = (R)reach * (R)reach;
+                        q.lim2 = (R)(reach * reach);
                         q.ct = pp.own ? (R)pp.ct : R(0);
 #pragma unroll
                         for (int a = 0; a < 3; ++a) {
@@ -495,32 +539,39 @@ __global__ void __launch_bounds__(TX *TY, (sizeof(typename P::real) == 4 && !MOV
         }
         [[maybe_unused]] const int nn = MOVING ? s_nn : 0;
         // component of a cell's offset to a particle, both in the domain: its minimum
-        // image (min_image's rule, without FP64: |d| < n, so one shift of the whole
-        // cells reaches it, before the one rounding)
-        [[maybe_unused]] auto wrapped = [](int d, R f, int n) -> R {
-            const R r = R(d) - f, half = R(0.5) * R(n);
-            if (r > half) return R(d - n) - f;
-            if (r < -half) return R(d + n) - f;
-            return r;
+        // image (min_image's rule; |d| < n, so one shift of the whole cells reaches it)
+        [[maybe_unused]] auto wrapped = [](int d, R fh, R fl, int n) -> Off<R> {
+            const R r = R(d) - fh, half = R(0.5) * R(n);
+            if (fabs(r) >= half) {
+                const Off<R> o = near_off<R>(d, fh, fl);
+                if (o.h > half || (o.h == half && o.l > R(0))) d -= n;
+                else if (o.h < -half || (o.h == -half && o.l < R(0))) d += n;
+            }
+            return near_off<R>(d, fh, fl);
         };
         // offset of cell (table cx, cy of the tile + 3 frame; plane z of the chunk's
         // run z0 - 2 ..) to near particle q, and its indicator there
         [[maybe_unused]] auto near_at = [&](const Near3<R> &q, int cx, int cy, int z, R &rx, R &ry, R &rz) -> R {
+            Off<R> ox, oy, oz;
             if (q.fast) {
-                rx = R(cx - 3 - q.ix) - q.fx;
-                ry = R(cy - 3 - q.iy) - q.fy;
-                rz = R(z - z0 - q.iz) - q.fz;
+                ox = near_off<R>(cx - 3 - q.i[0], q.fh[0], q.fl[0]);
+                oy = near_off<R>(cy - 3 - q.i[1], q.fh[1], q.fl[1]);
+                oz = near_off<R>(z - z0 - q.i[2], q.fh[2], q.fl[2]);
             } else {
-                rx = wrapped(s_gx[cx] - q.ix, q.fx, nx);
-                const int dy = s_gyi[cy] - q.iy;  // (no image across a wall)
-                ry = EXT && wall ? R(dy) - q.fy : wrapped(dy, q.fy, ny);
-                rz = wrapped(wrap_near(z, nz) - q.iz, q.fz, nz);
+                ox = wrapped(s_gx[cx] - q.i[0], q.fh[0], q.fl[0], nx);
+                const int dy = s_gyi[cy] - q.i[1];  // (no image across a wall)
+                oy = EXT && wall ? near_off<R>(dy, q.fh[1], q.fl[1]) : wrapped(dy, q.fh[1], q.fl[1], ny);
+                oz = wrapped(wrap_near(z, nz) - q.i[2], q.fh[2], q.fl[2], nz);
             }
-            return near_phi0_3d<R>(q, rx, ry, rz, (R)p.D);
+            rx = ox.h;
+            ry = oy.h;
+            rz = oz.h;
+            return near_phi0_3d<R>(q, ox, oy, oz, (R)p.D);
         };
         // whether near particle q may reach plane z (uniform)
         [[maybe_unused]] auto meets = [&](const Near3<R> &q, int z) -> bool {
-            const R dz = q.fast ? R(z - z0 - q.iz) - q.fz : wrapped(wrap_near(z, nz) - q.iz, q.fz, nz);
+            const R dz = q.fast ? near_off<R>(z - z0 - q.i[2], q.fh[2], q.fl[2]).h
+                                : wrapped(wrap_near(z, nz) - q.i[2], q.fh[2], q.fl[2], nz).h;
             return dz * dz < q.lim2;
         };
         // a tile whose frames reach beyond a wall

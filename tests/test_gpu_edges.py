@@ -366,3 +366,26 @@ def test_timed_out_step_leaves_outputs_alone(pf, monkeypatch, where):
             rc = pf.load().pf_get_macros(g._h, *[C.c_void_p(p[0]) for p in ptrs], w)
         assert rc == pf.PF_ETIMEOUT
         assert all(bool((b == 7.0).all()) for b in bufs)
+
+
+@pytest.mark.parametrize("shape,R", [((12, 10, 500), 200.0), ((112, 104, 128), 40.0)])
+def test_moving_3d_indicator_rounding_fp32(pf, shape, R):
+    """The particle's indicator in FP32 arithmetic: the squared distance of the FP64 offsets, rounded once (in a
+    box too small for one image, and in one wide enough).  At phi = 1 and 90 degrees mu_phi = c_pen phi0^2; the
+    bound is tanhf's and phi's roundings (2 ulp of 6e-8 each, the latter through c_dw and c_pen).  Distances in
+    FP32 throughout would differ by an ulp of R, 4e-6 and 1.5e-5."""
+    D, sigma = 1.0, 0.01
+    nz, ny, nx = shape
+    c = W.small_case(shape, seed=1, solid=False, D=D, theta_deg=90.0)
+    x = (0.5 * nx + 0.337, 0.5 * ny + 0.171, 0.5 * nz - 0.219)
+    g = pf.Sim(shape, precision="p32", **c["params"])
+    g.set_particle(0, x=x, R=R, rho_p=1.0)
+    g.init(np.zeros(shape), np.ones(shape))
+    mu = g.macros()["mu"] / (9.0 * sigma / D)
+    d = [np.arange(n) - v for n, v in zip((nx, ny, nz), x)]
+    dx, dy, dz = (v - n * np.rint(v / n) for v, n in zip(d, (nx, ny, nz)))
+    r2 = dx[None, None, :] ** 2 + dy[None, :, None] ** 2 + dz[:, None, None] ** 2
+    f = np.float32
+    z = f(2.0) * (f(R) - np.sqrt(r2.astype(f))) / f(D)
+    p0 = 0.5 * (1.0 + np.tanh(z.astype(np.float64)))
+    assert np.abs(mu - p0 * p0).max() <= 1e-6
