@@ -220,10 +220,11 @@ constexpr int step2d_min_blocks()
 // without it the wall code is compiled out (it costs registers)
 // UNIT: every domain of the launch has unit rates (DevParams::unit).  The order
 // parameter's populations are then only summed, the collisions take the short
-// forms above, and the four divisions of a cell become two.  In FP64 this is
-// what bounds the step: an SM retires two FP64 operations per cycle, and a cell
-// took about 540 of them (36 us per step of 128^2, 330 us for a batch of 0.27 M
-// cells).
+// forms above.  In FP64, where operations bound the step (an SM retires two per
+// cycle, and a cell took about 540 of them: 36 us per step of 128^2, 330 us for a
+// batch of 0.27 M cells), the four divisions of a cell also become two; FP32 keeps
+// four, each rounded once: shared ones saved 1% (512^2: 11.95 and 11.84 us per step)
+// and raised u's error after 32 steps with 16 particles from 3.3e-7 to 3.7e-7.
 template <class P, int TX, int TY, bool MOVING, int MODE, bool EXT, bool UNIT = false>
 __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY, UNIT && !MOVING && MODE == MODE_STEP>())) k_step2d(StepArgs A)
 {
@@ -714,13 +715,17 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY, UNIT && 
             sum_f = m3r + e24;
             jx = (f2[1] - f2[3]) + (d57 - d68);
             jy = (f2[2] - f2[4]) + (d57 + d68);
-            const R inv = R(1) / (rho * solid);  // one division for 1/rho and nu
-            irho = solid * inv;
-            nu = muv * inv;
+            if constexpr (sizeof(R) == 8) {
+                const R inv = R(1) / (rho * solid);  // one division for 1/rho and nu
+                irho = solid * inv;
+                nu = muv * inv;
+            }
         } else {
             jx = f2[1] - f2[3] + f2[5] - f2[6] - f2[7] + f2[8];
             jy = f2[2] - f2[4] + f2[5] + f2[6] - f2[7] - f2[8];
             sum_f = f2[1] + f2[2] + f2[3] + f2[4] + f2[5] + f2[6] + f2[7] + f2[8];
+        }
+        if constexpr (!UNIT || sizeof(R) == 4) {
             irho = R(1) / rho;
             nu = muv / (rho * solid);
         }
@@ -804,8 +809,15 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY, UNIT && 
                 collide9_unit_phi<R>(f1, phi, pux + R(0.5) * (pux - php * upx), puy + R(0.5) * (puy - php * upy),
                                      ku.c2eta * mu, ku);
                 // flow (Eqs. 32-34): second-order equilibria and sources
-                const R inv_ab = R(1) / (inv_s2a * inv_s2b);  // one division for both rates
-                const R s2a = inv_s2b * inv_ab, s2b = inv_s2a * inv_ab;
+                R s2a, s2b;
+                if constexpr (sizeof(R) == 8) {
+                    const R inv_ab = R(1) / (inv_s2a * inv_s2b);  // one division for both rates
+                    s2a = inv_s2b * inv_ab;
+                    s2b = inv_s2a * inv_ab;
+                } else {
+                    s2a = R(1) / inv_s2a;
+                    s2b = R(1) / inv_s2b;
+                }
                 const R m0 = f2[0] + sum_f, c3u = ku.c3 * ugr;
                 const R cross = Sx * uy + ux * Sy, crossp = Spx * upy + upx * Spy;
                 const R d3 = m3r - ku.cs2 * m0, d4 = m4r - ku.cs2 * m0;
