@@ -389,3 +389,30 @@ def test_moving_3d_indicator_rounding_fp32(pf, shape, R):
     z = f(2.0) * (f(R) - np.sqrt(r2.astype(f))) / f(D)
     p0 = 0.5 * (1.0 + np.tanh(z.astype(np.float64)))
     assert np.abs(mu - p0 * p0).max() <= 1e-6
+
+
+def _finish(nx, ny, seg, places=304, band=4):
+    """When the last of a domain's strip items ends, in rows, handed out longest first to the chip's places."""
+    import heapq
+    strips = (nx + 63) // 64
+    rows = [seg] * (strips * (ny // seg)) + [ny % seg] * (strips if ny % seg else 0)
+    load = [0] * places
+    for r in rows:
+        heapq.heapreplace(load, load[0] + (r + band - 1) // band * band + 10)
+    return max(load)
+
+
+def test_strip_segment_of_other_sizes(pf):
+    """The segment length tuned on one domain is not taken over by another size of the same cell-count class:
+    that one's items end within a tenth of the earliest, as the tuned ones do (56 rows of 692 x 761: 1.74)."""
+    for shape in ((1024, 1024), (761, 692), (940, 1100), (600, 1000)):
+        c = W.small_case(shape, seed=1, solid=False)
+        s = pf.Sim(shape, precision="p32", walls_y=True, **c["params"])
+        s.init(c["phi0"], np.ones(shape))
+        s.autotune()
+        tx, seg, _, kernel = s.config()
+        if kernel != 4:
+            continue
+        ny, nx = shape
+        best = min(_finish(nx, ny, k) for k in range(8, 260, 4))
+        assert _finish(nx, ny, seg) <= 1.1 * best, (shape, seg)
