@@ -9,7 +9,6 @@
 #include <cstdlib>
 #include <cstring>
 #include <map>
-#include <queue>
 #include <mutex>
 #include <string>
 #include <tuple>
@@ -1019,16 +1018,17 @@ static int strip_setup(Engine &E, int seg)
 // The segment lengths worth timing: those whose items, handed out longest first,
 // finish earliest on the chip's two CTAs per SM by a count of rows (an item takes
 // its rows, in whole bands, and a prologue worth about ten).  1024 x 1024: 56 rows
-// make 304 items for 304 places, 51.1 us per step; 64 rows 256 items, 54.8 us; 48
-// rows 352 items, 73.7 us.
+// make 304 items for 304 places, 47.7 us per step; 64 rows 256 items, 51.1 us; 72
+// rows 55.2.  Lengths are whole bands, a band apart up to 16 bands and two beyond:
+// a finer step there is less than what the count misses by (64 sweep domains in
+// FP16: 204 rows end at 224 and 108 at 236, and take 125.0 and 122.6 us).
 static void strip_segments(const Engine &E, int *out, int n)
 {
-    static const int cand[] = {8, 12, 16, 20, 24, 28, 32, 36, 40, 48, 54, 56, 60, 64, 72, 80, 84, 96, 102, 108, 120, 128, 144, 160, 168, 192, 216, 256};
     const int B = E.prec == PF_P32 ? 4 : 6;
     std::vector<std::pair<long long, int>> rank;
     int nymax = 0, before = 0;
     for (auto &m : E.mem) nymax = std::max(nymax, m.d.ny);
-    for (int seg : cand) {
+    for (int seg = 2 * B; seg <= 256; seg += seg < 16 * B ? B : 2 * B) {
         if (before >= nymax) break;  // (one segment per strip from there on)
         before = seg;
         std::map<int, long long, std::greater<int>> items;  // rows -> count
@@ -1037,32 +1037,19 @@ static void strip_segments(const Engine &E, int *out, int n)
             if (m.d.ny / seg) items[seg] += strips * (m.d.ny / seg);
             if (m.d.ny % seg) items[m.d.ny % seg] += strips;
         }
-        // (equal items fill the places in rounds; the places are a heap by load)
-        std::priority_queue<long long, std::vector<long long>, std::greater<long long>> load;
-        for (int k = 0; k < 2 * E.nsm; ++k) load.push(0);
-        long long last = 0;
+        // the places by load: equal items go to all places of the least load at once
+        std::map<long long, long long> load{{0, 2 * E.nsm}};
         for (auto &it : items) {
             const long long c = (it.first + B - 1) / B * B + 10;
-            long long left = it.second;
-            const long long rounds = left / (2 * E.nsm) > 4 ? left / (2 * E.nsm) - 4 : 0;
-            if (rounds) {  // whole rounds raise every place alike
-                std::priority_queue<long long, std::vector<long long>, std::greater<long long>> q;
-                while (!load.empty()) {
-                    q.push(load.top() + rounds * c);
-                    last = std::max(last, load.top() + rounds * c);
-                    load.pop();
-                }
-                load.swap(q);
-                left -= rounds * 2 * E.nsm;
-            }
-            for (; left > 0; --left) {
-                const long long v = load.top() + c;
-                load.pop();
-                load.push(v);
-                last = std::max(last, v);
+            for (long long left = it.second; left > 0;) {
+                const auto least = load.begin();
+                const long long v = least->first, k = std::min(least->second, left);
+                if ((least->second -= k) == 0) load.erase(least);
+                load[v + c] += k;
+                left -= k;
             }
         }
-        rank.push_back({last, -seg});  // (ties: the longer segment)
+        rank.push_back({load.rbegin()->first, -seg});  // (ties: the longer segment)
     }
     std::sort(rank.begin(), rank.end());
     for (int k = 0; k < n; ++k) out[k] = -rank[std::min<size_t>(k, rank.size() - 1)].second;
