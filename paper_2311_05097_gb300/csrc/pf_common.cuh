@@ -278,8 +278,7 @@ struct StepArgs {
     int wait_polls;        // polls of one bounded device wait (staged kernel); 0: default
     const unsigned char *tile_sel;  // optional, per tile in device memory: run only the tiles ...
     int sel;                        // ... whose byte equals sel (else every tile)
-    int pdl;               // single-cell step without particles: one tile per CTA, all resident at once
-                           // (the launch overlaps the step before it)
+    int pdl;               // single-cell step without particles: launch it over the step before
     int *queue;            // strip step: work-queue counter (0 at the launch, and left at 0), or
                            // null: static round-robin over the items
     int mu0;               // single-cell step, wall instantiation, no particle terms: the

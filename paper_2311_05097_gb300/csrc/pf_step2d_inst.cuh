@@ -21,8 +21,7 @@ static bool run2d(int grid, cudaStream_t s, const StepArgs &a, int *occ)
         return true;
     }
     if constexpr (MODE == MODE_STEP) {
-        // after the particle update, or where all CTAs are resident at once: a launch of
-        // several waves gains nothing and ran up to 4% longer (1024 x 1000).  Not the
+        // after the particle update, or where StepArgs::pdl says that it pays.  Not the
         // split step, whose two launches run on two streams.
         if (!a.tile_sel && (MOVING || a.pdl)) {
             launch_pdl(kern, grid, TX * TY, 0, s, a);

@@ -416,3 +416,24 @@ def test_strip_segment_of_other_sizes(pf):
         ny, nx = shape
         best = min(_finish(nx, ny, k) for k in range(8, 260, 4))
         assert _finish(nx, ny, seg) <= 1.1 * best, (shape, seg)
+
+
+# 32 x 8 tiles: 64 (one per SM or fewer), 300 (two), 352 (three: not overlapped), 512 (four), 640 (two waves)
+@pytest.mark.parametrize("ny", [64, 300, 352, 512, 640])
+@pytest.mark.parametrize("precision,walls", [("p32", False), ("fp16", False), ("fp16", True), ("p64", True)])
+def test_overlapped_steps_equal_waited_ones(pf, ny, precision, walls):
+    """The single-cell step launched over the step before it, where the rule says so, and steps waited for one by
+    one: the same bits."""
+    shape = (ny, 250)
+    c = W.small_case(shape, seed=2, solid=True, u_amp=0.01, rho_ratio=2.0, mu_ratio=2.0)
+    sims = []
+    for _ in range(2):
+        s = pf.Sim(shape, precision=precision, walls_y=walls, **c["params"])
+        s.init(c["phi0"], c["phi"], c["u"])
+        sims.append(s)
+    sims[0].step(20)
+    for _ in range(20):
+        sims[1].step(1)
+        sims[1].sync()
+    a, b = sims[0].macros(), sims[1].macros()
+    assert all(np.array_equal(a[k], b[k]) for k in a)
