@@ -216,6 +216,17 @@ constexpr int step2d_min_blocks()
     return P::id == 0 ? (CAP64 ? 512 / (TX * TY) : 1) : (TX * TY > 256 ? 2 : ((TX == 32 && TY == 8) ? 4 : 3));
 }
 
+// Whether an instantiation may be launched over the step before it (see pdl_begin;
+// its loads are then plain ones).  Not the 16-bit ones with the wall and Allen-Cahn
+// code at general rates, which run faster through the read-only path: 700 x 700 in
+// FP16 with walls 30.3 us per step, 32.4 with plain loads; 64 x 64 7.1, and 7.3
+// overlapped.
+template <class P, bool MOVING, bool EXT, bool UNIT>
+constexpr bool step2d_dependent()
+{
+    return MOVING || UNIT || !(EXT && P::MIX);
+}
+
 // EXT: the instantiation also handles domains with walls at the ends of y;
 // without it the wall code is compiled out (it costs registers)
 // UNIT: every domain of the launch has unit rates (DevParams::unit).  The order
@@ -264,12 +275,17 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY, UNIT && 
     // w_z, cos(own angle) (0 without one)
     __shared__ R s_pv[MOVING ? PMAX : 1][6];
 
+    constexpr bool DEP = step2d_dependent<P, MOVING, EXT, UNIT>();
+    auto ld = [](const auto *p) {
+        if constexpr (DEP) return ldp(p);
+        else return ldg(p);
+    };
     const int tid = threadIdx.x;
     const int lx = tid % TX, ly = tid / TX;
     // a step that timed out (bit 2) leaves no fields to read: nothing is written
     [[maybe_unused]] int lost = 0;
     if constexpr (MODE == MODE_MACROS) lost = *A.flags & 4;
-    if constexpr (MODE == MODE_STEP) pdl_begin();
+    if constexpr (MODE == MODE_STEP && DEP) pdl_begin();
 
     for (int t = blockIdx.x; t < A.ntiles; t += gridDim.x) {
         if (A.tile_sel && A.tile_sel[t] != A.sel) continue;  // (uniform in the block)
@@ -387,7 +403,10 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY, UNIT && 
             return base * plane + i * plane + s_gy[cy - CY9[i]] + s_gx[cx - CX9[i]];
         };
 
-        // phi at frame cell (hx, hy) of the tile+2 frame: pull and sum (Eq. 31)
+        // phi at frame cell (hx, hy) of the tile+2 frame: pull and sum (Eq. 31).  Every
+        // load before the first addition: summed as they were loaded, the branches of
+        // the wall pulls kept each load behind the sum of those before it (700 x 700 with
+        // walls, us per step: FP32 38.3 and 27.8, FP16 36.1 and 26.5)
         long long rest_own = 0;
         auto phi_at = [&](int hx, int hy, R *keep, ST *keepq) -> R {
             const int cx = hx + 1, cy = hy + 1;  // tile+3 table coordinates
@@ -397,21 +416,26 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY, UNIT && 
                 acc = float_of_fixed(rv);
                 if (keep) keep[0] = acc;
                 if (keepq) rest_own = rv;
+                ST q[9];
+#pragma unroll
+                for (int i = 1; i < 9; ++i) q[i] = ld(fs + pull(0, i, cx, cy));
                 R movers = R(0);  // sum in stored units, scaled once
 #pragma unroll
                 for (int i = 1; i < 9; ++i) {
-                    ST q = ldp(fs + pull(0, i, cx, cy));
-                    const R v = stored_to_float<ST>(q);
+                    const R v = stored_to_float<ST>(q[i]);
                     if (keep) keep[i] = v * isc1;
-                    if (keepq) keepq[i] = q;
+                    if (keepq) keepq[i] = q[i];
                     movers += v;
                 }
                 acc += movers * isc1;
             } else {
+                ST q[9];
+#pragma unroll
+                for (int i = 0; i < 9; ++i) q[i] = ld(fs + pull(0, i, cx, cy));
                 acc = R(0);
 #pragma unroll
                 for (int i = 0; i < 9; ++i) {
-                    R v = Conv<P>::ld(ldp(fs + pull(0, i, cx, cy)), isc1);
+                    const R v = Conv<P>::ld(q[i], isc1);
                     if (keep) keep[i] = v;
                     acc += v;
                 }
@@ -424,7 +448,7 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY, UNIT && 
         // indicator at this cell is not 0
         auto phi0_at = [&](int hx, int hy, [[maybe_unused]] unsigned long long &hits) -> R {
             const int cx = hx + 1, cy = hy + 1;
-            R v = (R)ldp(ph0 + s_gy[cy] + s_gx[cx]);
+            R v = (R)ld(ph0 + s_gy[cy] + s_gx[cx]);
             any_solid |= v != R(0);
             if constexpr (MOVING) {
                 const int gx = s_gx[cx], gy = s_gyi[cy];
@@ -461,11 +485,11 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY, UNIT && 
         const int id = s_gy[ly + 3] + s_gx[lx + 3];
         ST f2raw[9];
 #pragma unroll
-        for (int i = 0; i < 9; ++i) f2raw[i] = ldp(fs + pull(9, i, lx + 3, ly + 3));
+        for (int i = 0; i < 9; ++i) f2raw[i] = ld(fs + pull(9, i, lx + 3, ly + 3));
         AX lag[5];
         if constexpr (MODE == MODE_STEP) {
 #pragma unroll
-            for (int k = 0; k < 5; ++k) lag[k] = ldp(as + k * plane + id);
+            for (int k = 0; k < 5; ++k) lag[k] = ld(as + k * plane + id);
         }
         R f1[9];
         ST q1[9];
@@ -520,8 +544,8 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY, UNIT && 
                     wx = (rr & 1) ? TX + 1 : 0;
                 }
                 const int wid = s_gy[wy + 2] + s_gx[wx + 2];
-                const R ux = (R)ldp(as + 0 * plane + wid), uy = (R)ldp(as + 1 * plane + wid);
-                const R Sx = (R)ldp(as + 2 * plane + wid), Sy = (R)ldp(as + 3 * plane + wid);
+                const R ux = (R)ld(as + 0 * plane + wid), uy = (R)ld(as + 1 * plane + wid);
+                const R Sx = (R)ld(as + 2 * plane + wid), Sy = (R)ld(as + 3 * plane + wid);
                 s_w[wy][wx] = wsign(wy + 2) * (Sx * uy - ux * Sy);
             }
         }
@@ -684,8 +708,8 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY, UNIT && 
 #pragma unroll
                 for (int i = -1; i <= 1; ++i) {
                     const int nid = s_gy[ly + 3 + j] + s_gx[lx + 3 + i];
-                    const R ux = (R)ldp(as + 0 * plane + nid), uy = (R)ldp(as + 1 * plane + nid);
-                    const R sx = (R)ldp(as + 2 * plane + nid), sy = (R)ldp(as + 3 * plane + nid);
+                    const R ux = (R)ld(as + 0 * plane + nid), uy = (R)ld(as + 1 * plane + nid);
+                    const R sx = (R)ld(as + 2 * plane + nid), sy = (R)ld(as + 3 * plane + nid);
                     wv[j + 1][i + 1] = wsign(ly + 3 + j) * (sx * uy - ux * sy);
                 }
             R wgx, wgy;
@@ -750,7 +774,7 @@ __global__ void __launch_bounds__(TX *TY, (step2d_min_blocks<P, TX, TY, UNIT && 
         // macroscopic pass reads them here)
         if constexpr (MODE == MODE_MACROS) {
 #pragma unroll
-            for (int k = 0; k < 5; ++k) lag[k] = ldp(as + k * plane + id);
+            for (int k = 0; k < 5; ++k) lag[k] = ld(as + k * plane + id);
         }
         const R upx = (R)lag[0], upy = (R)lag[1];
         const R Spx = (R)lag[2], Spy = (R)lag[3];

@@ -20,7 +20,7 @@ static bool run2d(int grid, cudaStream_t s, const StepArgs &a, int *occ)
         *occ = n;
         return true;
     }
-    if constexpr (MODE == MODE_STEP) {
+    if constexpr (MODE == MODE_STEP && step2d_dependent<P, MOVING, EXT, UNIT>()) {
         // after the particle update, or where StepArgs::pdl says that it pays.  Not the
         // split step, whose two launches run on two streams.
         if (!a.tile_sel && (MOVING || a.pdl)) {
