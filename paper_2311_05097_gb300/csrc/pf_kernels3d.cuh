@@ -293,66 +293,46 @@ __device__ __forceinline__ const DomainDev &tile_of(const StepArgs &A, const Dom
 // the plane of phi of the step under way (k_phi3d)
 __device__ __forceinline__ float *phi_of_step(const DomainDev &Dm) { return reinterpret_cast<float *>(Dm.phi0) + Dm.plane; }
 
-// One particle near a tile: its centre as whole cells i and a fraction in two
-// parts of the arithmetic type (fh + fl: FP64 holds it in fh alone, two FP32
-// parts to 48 bits).  fast: the whole cells are those of the image nearest to the
-// tile, in the tile's coordinates, and serve every cell of its frames.  Otherwise
-// (the box is too small for one image, or the frames hold mirror rows) they are
-// the domain's, 0 .. n - 1, and each cell takes its minimum image from its own
-// wrapped coordinates: a table coordinate may lie several lengths of a box
-// narrower than the tile from the image.
+// One particle near a tile: its centre as the nearest whole cell i and the rest
+// f = fh + fl, |f| <= 1/2, in two parts of the arithmetic type (FP64: fh alone; FP32:
+// fh in steps of 2^-16 and fl), f2 = |f|^2.  fast: the whole cells are those of the
+// image nearest to the tile, in the tile's coordinates, and serve every cell of its
+// frames.  Otherwise (the box is too small for one image, or the frames hold mirror
+// rows) they are the domain's, and each cell takes its minimum image from its own
+// wrapped coordinates: a table coordinate may lie several lengths of a box narrower
+// than the tile from the image.
 template <class R>
 struct Near3 {
     int i[3], k, own, fast;
-    R fh[3], fl[3], Rp, lim2, ct;
+    R fh[3], fl[3], f2, Rp, lim2, ct;
     R u[3], w[3];
 };
 
-// A component of a cell's offset, d - f for whole cells d: h is the difference
-// rounded once, h + l the difference (FP32: to 2^-48; FP64: l = 0).
+// Indicator of a cell d whole cells from the particle's (offset d - f).  FP32: the
+// squared distance is |d|^2 - 2 d.f + f2, where |d|^2 and d.fh are exact (for
+// |d| < 128; beyond, far within the result's rounding), their difference carries its
+// error and the other terms are small, so it is rounded once, as that of FP64
+// arithmetic is, whose pipe (two lanes per SM and clock) stays free.  Three
+// placements of three spheres in 96 x 80 x 112: 189, 210 and 226 us per step; with
+// plain FP32 sums, an ulp of R off in the distance, 189, 211 and 227.
 template <class R>
-struct Off {
-    R h, l;
-};
-template <class R>
-__device__ __forceinline__ Off<R> near_off(int d, R fh, R fl)
+__device__ __forceinline__ R near_phi0_3d(const Near3<R> &q, const int (&d)[3], R D)
 {
-    const R a = R(d), s = a - fh;
-    if constexpr (sizeof(R) == 8) return {s, R(0)};
-    const R e = ((a - s) - fh) - fl;  // (a - s) - fh is exact: |a| >= fh or a = 0
-    const R h = s + e;
-    return {h, e - (h - s)};
-}
-
-// Indicator at an offset.  FP32: the squares and their sum carry their rounding
-// errors (two-term products and sums), so the squared distance is rounded once, as
-// that of FP64 arithmetic is, whose pipe (two lanes per SM and clock) stays free.
-// Three placements of three spheres in 96 x 80 x 112: 194, 209 and 232 us per step;
-// with plain FP32 sums, an ulp of R off in the distance, 189, 211 and 227.
-template <class R>
-__device__ __forceinline__ R near_phi0_3d(const Near3<R> &q, Off<R> x, Off<R> y, Off<R> z, R D)
-{
-    // (FP32: the indicator is 0 well inside this sum's roundings of the limit, so it
-    // decides the reach)
-    R r2 = x.h * x.h + y.h * y.h + z.h * z.h;
-    if (r2 >= q.lim2) return R(0);
-    if constexpr (sizeof(R) == 4) {
-        auto square = [](Off<R> o, R &err) -> R {
-            const R p = __fmul_rn(o.h, o.h);
-            err = __fmaf_rn(o.h + o.h, o.l, __fmaf_rn(o.h, o.h, -p));
-            return p;
-        };
-        auto add = [](R a, R b, R &err) -> R {
-            const R s = a + b, t = s - a;
-            err += (a - (s - t)) + (b - t);
-            return s;
-        };
-        R ex, ey, ez;
-        const R px = square(x, ex), py = square(y, ey), pz = square(z, ez);
-        R err = (ex + ey) + ez;
-        const R s = add(add(px, py, err), pz, err);
-        r2 = s + err;
+    const R x = R(d[0]), y = R(d[1]), z = R(d[2]);
+    R r2;
+    if constexpr (sizeof(R) == 8) {
+        const R rx = x - q.fh[0], ry = y - q.fh[1], rz = z - q.fh[2];
+        r2 = rx * rx + ry * ry + rz * rz;
+    } else {
+        const R whole = __fmaf_rn(z, z, __fmaf_rn(y, y, __fmul_rn(x, x)));
+        const R dh = __fmaf_rn(z, q.fh[2], __fmaf_rn(y, q.fh[1], __fmul_rn(x, q.fh[0])));
+        const R dl = __fmaf_rn(z, q.fl[2], __fmaf_rn(y, q.fl[1], __fmul_rn(x, q.fl[0])));
+        // (|d|^2 >= |2 d.fh|: d are whole numbers and |fh| <= 1/2, so err is exact)
+        const R s = __fmaf_rn(R(-2), dh, whole);
+        const R err = __fmaf_rn(R(-2), dh, whole - s);
+        r2 = s + (err + __fmaf_rn(R(-2), dl, q.f2));
     }
+    if (r2 >= q.lim2) return R(0);
     return R(0.5) * (R(1) + tanh(R(2) * (q.Rp - sqrt(r2)) / D));
 }
 
@@ -491,7 +471,7 @@ __global__ void __launch_bounds__(TX *TY, (sizeof(typename P::real) == 4 && !MOV
                         const double ext[3] = {0.5 * TX + 2.0, 0.5 * TY + 2.0, 0.5 * zc + 2.0};
                         const int n3[3] = {nx, ny, nz}, len[3] = {TX, TY, zc};
                         const double reach = pp.R + indicator_cut<R>(p);
-                        double e2 = 0.0, cell[3];
+                        double e2 = 0.0, f2 = 0.0, cell[3];
                         bool fast = true;
 #pragma unroll
                         for (int a = 0; a < 3; ++a) {
@@ -502,10 +482,11 @@ __global__ void __launch_bounds__(TX *TY, (sizeof(typename P::real) == 4 && !MOV
                             dd -= shift;
                             const double ex = fmax(fabs(dd) - ext[a], 0.0);
                             e2 += ex * ex;
-                            const double whole = floor(pp.x[a]), frac = pp.x[a] - whole;
+                            const double whole = rint(pp.x[a]), f = pp.x[a] - whole;
                             cell[a] = whole + shift;
-                            q.fh[a] = (R)frac;
-                            q.fl[a] = (R)(frac - (double)q.fh[a]);
+                            f2 += f * f;
+                            q.fh[a] = sizeof(R) == 8 ? (R)f : (R)(rint(f * 65536.0) / 65536.0);
+                            q.fl[a] = (R)(f - (double)q.fh[a]);
                             // with walls rows beyond them are mirror rows: their cells are not
                             // where the table says
                             fast = fast && (bounded ? !(y0 - 3 < 0 || y0 + TY + 3 > ny) : n3[a] >= 2.0 * reach + 6.0 + len[a]);
@@ -516,6 +497,7 @@ __global__ void __launch_bounds__(TX *TY, (sizeof(typename P::real) == 4 && !MOV
                         for (int a = 0; a < 3; ++a)
                             q.i[a] = fast ? (int)cell[a] - at[a]
                                           : (a == 1 && wall ? (int)cell[a] : wrap_idx((int)cell[a], n3[a]));
+                        q.f2 = (R)f2;
                         q.k = k;
                         q.own = pp.own;
                         q.fast = fast;
@@ -538,40 +520,39 @@ __global__ void __launch_bounds__(TX *TY, (sizeof(typename P::real) == 4 && !MOV
             __syncthreads();
         }
         [[maybe_unused]] const int nn = MOVING ? s_nn : 0;
-        // component of a cell's offset to a particle, both in the domain: its minimum
-        // image (min_image's rule; |d| < n, so one shift of the whole cells reaches it)
-        [[maybe_unused]] auto wrapped = [](int d, R fh, R fl, int n) -> Off<R> {
-            const R r = R(d) - fh, half = R(0.5) * R(n);
-            if (fabs(r) >= half) {
-                const Off<R> o = near_off<R>(d, fh, fl);
-                if (o.h > half || (o.h == half && o.l > R(0))) d -= n;
-                else if (o.h < -half || (o.h == -half && o.l < R(0))) d += n;
-            }
-            return near_off<R>(d, fh, fl);
+        // whole cells d of an offset d - f within the domain (component a of particle q):
+        // those of its minimum image (min_image's rule; |d| < n, so one shift reaches it)
+        [[maybe_unused]] auto wrapped = [](const Near3<R> &q, int a, int d, int n) -> int {
+            const R fh2 = R(2) * q.fh[a], fl2 = R(2) * q.fl[a];  // (exact, as the differences are)
+            if (R(2 * d - n) - fh2 > fl2) return d - n;
+            if (R(2 * d + n) - fh2 < fl2) return d + n;
+            return d;
         };
-        // offset of cell (table cx, cy of the tile + 3 frame; plane z of the chunk's
-        // run z0 - 2 ..) to near particle q, and its indicator there
+        // whole cells of the offset of plane z (of the chunk's run z0 - 2 ..) to particle q
+        [[maybe_unused]] auto near_z = [&](const Near3<R> &q, int z) -> int {
+            return q.fast ? z - z0 - q.i[2] : wrapped(q, 2, wrap_near(z, nz) - q.i[2], nz);
+        };
+        // offset of cell (table cx, cy of the tile + 3 frame, plane z) to near particle q,
+        // rounded once, and its indicator there
         [[maybe_unused]] auto near_at = [&](const Near3<R> &q, int cx, int cy, int z, R &rx, R &ry, R &rz) -> R {
-            Off<R> ox, oy, oz;
+            int d[3];
+            d[2] = near_z(q, z);
             if (q.fast) {
-                ox = near_off<R>(cx - 3 - q.i[0], q.fh[0], q.fl[0]);
-                oy = near_off<R>(cy - 3 - q.i[1], q.fh[1], q.fl[1]);
-                oz = near_off<R>(z - z0 - q.i[2], q.fh[2], q.fl[2]);
+                d[0] = cx - 3 - q.i[0];
+                d[1] = cy - 3 - q.i[1];
             } else {
-                ox = wrapped(s_gx[cx] - q.i[0], q.fh[0], q.fl[0], nx);
-                const int dy = s_gyi[cy] - q.i[1];  // (no image across a wall)
-                oy = EXT && wall ? near_off<R>(dy, q.fh[1], q.fl[1]) : wrapped(dy, q.fh[1], q.fl[1], ny);
-                oz = wrapped(wrap_near(z, nz) - q.i[2], q.fh[2], q.fl[2], nz);
+                d[0] = wrapped(q, 0, s_gx[cx] - q.i[0], nx);
+                d[1] = s_gyi[cy] - q.i[1];  // (no image across a wall)
+                if (!(EXT && wall)) d[1] = wrapped(q, 1, d[1], ny);
             }
-            rx = ox.h;
-            ry = oy.h;
-            rz = oz.h;
-            return near_phi0_3d<R>(q, ox, oy, oz, (R)p.D);
+            rx = (R(d[0]) - q.fh[0]) - q.fl[0];
+            ry = (R(d[1]) - q.fh[1]) - q.fl[1];
+            rz = (R(d[2]) - q.fh[2]) - q.fl[2];
+            return near_phi0_3d<R>(q, d, (R)p.D);
         };
         // whether near particle q may reach plane z (uniform)
         [[maybe_unused]] auto meets = [&](const Near3<R> &q, int z) -> bool {
-            const R dz = q.fast ? near_off<R>(z - z0 - q.i[2], q.fh[2], q.fl[2]).h
-                                : wrapped(wrap_near(z, nz) - q.i[2], q.fh[2], q.fl[2], nz).h;
+            const R dz = (R(near_z(q, z)) - q.fh[2]) - q.fl[2];
             return dz * dz < q.lim2;
         };
         // a tile whose frames reach beyond a wall
