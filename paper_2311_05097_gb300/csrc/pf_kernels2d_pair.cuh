@@ -579,11 +579,12 @@ __device__ __forceinline__ void pair_cells(const StepArgs &A, const DevParams &p
 #pragma unroll
             for (int i = 0; i < 9; ++i) fd[(9 + i) * plane + idc] = half(w2[i]);
         } else {
+            // (one lattice after the other: alternating between them took 28.3 us per step
+            // of 700 x 700 in 32 x 16 tiles, Allen-Cahn, and this 26.7)
 #pragma unroll
-            for (int i = 0; i < 9; ++i) {
-                fd[i * plane + idc] = Conv<P>::st(c == 0 ? f1[i].v.x : f1[i].v.y, 1.0f);
-                fd[(9 + i) * plane + idc] = Conv<P>::st(c == 0 ? f2[i].v.x : f2[i].v.y, 1.0f);
-            }
+            for (int i = 0; i < 9; ++i) fd[i * plane + idc] = Conv<P>::st(c == 0 ? f1[i].v.x : f1[i].v.y, 1.0f);
+#pragma unroll
+            for (int i = 0; i < 9; ++i) fd[(9 + i) * plane + idc] = Conv<P>::st(c == 0 ? f2[i].v.x : f2[i].v.y, 1.0f);
         }
         // fields of this step, read as the previous step's by the next one
         ad[0 * plane + idc] = (AX)uxc;
