@@ -477,10 +477,11 @@ def run_batch(args, dist, rank, world, local):
                 kernel=step_kernel_name(2, cpt), launch_config=[tx, ty, cpt])
 
 
-def step_kernel_name(dim, variant):
-    """The step kernel(s) of a launch variant (the roofline's dominant kernel)."""
+def step_kernel_name(dim, variant, prec="", particles=False):
+    """The step kernel(s) of a launch variant (the roofline's dominant kernel).  3D: FP32 arithmetic sums phi in
+    a pass of its own, and without particles updates two cells per thread."""
     if dim == 3:
-        return "k_step3d"
+        return "k_step3d" if prec == "p64" else "k_phi3d+k_step3d" if particles else "k_phi3d+k_step3d_pair"
     return ["k_step2d", "k_step2d_pair", "k_step2d_stage", "k_step2d_pair+k_step2d", "k_step2d_strip"][variant]
 
 
@@ -687,30 +688,36 @@ def run_single_large(args, dist, rank, world, local, case, prec, cells, bpc, sim
            "l2": "state (%.2f GB) larger than L2 (129 MB); no flush" % (cells * bpc / 1e9), **launch,
            "kernels_per_step": nker,
            "parallelism": "independent replicas per GPU" if world > 1 else "single GPU"}
-    kernel = step_kernel_name(len(case["shape"]), launch["kernel"])
+    kernel = step_kernel_name(len(case["shape"]), launch["kernel"], prec, bool(case.get("particles")))
     return dict(mlups=mlups, total_ms=total_ms, achieved=achieved, bpc=bpc, prec=prec, cfg=cfg,
                 clk=clk, launches=launches, e2e=e2e, t_wall=t_wall, kernel=kernel)
 
 
-# FP64 instructions per 2D cell update of the FP64 step at unit rates (DADD + DMUL +
-# DFMA thread instructions per cell from ncu on a batch of drops on a wall, kernel 0)
-FP64_INST_PER_CELL_2D = 275.1
+# FP64 instructions per 2D cell update of the FP64 step (kernel 0: DADD + DMUL + DFMA thread instructions per
+# cell, ncu) of the workloads it was counted on: (workload, phase model).  The count depends on the rates, the
+# tile, the solids and the walls: other runs report the HBM fraction only.
+FP64_INST_PER_CELL_2D = {("static_drop", 0): 244.2,  # unit rates, 16 x 8 blocks, no solid
+                         ("static_drop", 1): 451.8,  # general collisions (Allen-Cahn)
+                         ("batch", 0): 247.8}        # unit rates, 32 x 8 tiles, wall slabs
 GB300_SMS = 152
 FP64_INST_PER_CLK_PER_SM = 2  # DFMA/DADD/DMUL issue rate of one SM (ncu peak_sustained)
 
 
 def roofline_entry(args, r, peak, peak_src):
     """HBM roofline of the step; the FP64 2D step is bound by the FP64 pipe
-    instead: achieved FP64 instructions per second against the pipe's rate at
-    the SM clock measured during the timed region."""
-    dim3 = r["kernel"] == "k_step3d"
-    if r["prec"] == "p64" and not dim3:
+    instead: achieved FP64 instructions per second (where they have been
+    counted) against the pipe's rate at the SM clock measured during the timed
+    region."""
+    count = FP64_INST_PER_CELL_2D.get((args.workload, args.phase_model))
+    if args.workload == "batch" and args.batch_count < 64:
+        count = None  # (fewer domains may run as 16 x 8 blocks)
+    if r["prec"] == "p64" and r["kernel"] == "k_step2d" and count:
         mhz = (r.get("clk") or {}).get("sm_mhz") or 2070.0
         peak_i = GB300_SMS * FP64_INST_PER_CLK_PER_SM * mhz * 1e-3  # G instructions / s
-        ach = FP64_INST_PER_CELL_2D * r["mlups"] * 1e-3
+        ach = count * r["mlups"] * 1e-3
         return {"bound": "alu", "achieved": round(ach, 1), "peak": round(peak_i, 1),
                 "unit": "G FP64 inst/s", "frac": round(ach / peak_i, 4), "traffic": None,
-                "fp64_inst_per_cell": FP64_INST_PER_CELL_2D, "kernel": r["kernel"],
+                "fp64_inst_per_cell": count, "kernel": r["kernel"],
                 "peak_source": "152 SMs x 2 FP64 instructions/clock x SM clock (unit counts and clocks)",
                 "hbm_frac": round(r["achieved"] / peak, 4)}
     return {"bound": "hbm", "achieved": round(r["achieved"], 1), "peak": peak,
