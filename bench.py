@@ -694,11 +694,12 @@ def run_single_large(args, dist, rank, world, local, case, prec, cells, bpc, sim
 
 
 # FP64 instructions per 2D cell update of the FP64 step (kernel 0: DADD + DMUL + DFMA thread instructions per
-# cell, ncu) of the workloads it was counted on: (workload, phase model).  The count depends on the rates, the
+# cell, ncu) of the runs it was counted on: (workload, phase model, tile).  The count depends on the rates, the
 # tile, the solids and the walls: other runs report the HBM fraction only.
-FP64_INST_PER_CELL_2D = {("static_drop", 0): 244.2,  # unit rates, 16 x 8 blocks, no solid
-                         ("static_drop", 1): 451.8,  # general collisions (Allen-Cahn)
-                         ("batch", 0): 247.8}        # unit rates, 32 x 8 tiles, wall slabs
+FP64_INST_PER_CELL_2D = {("static_drop", 0, (32, 8)): 244.2,  # unit rates, no solid (as 16 x 8 blocks)
+                         ("static_drop", 1, (32, 8)): 451.8,  # general collisions (Allen-Cahn)
+                         ("batch", 0, (32, 8)): 247.8,        # unit rates, wall slabs
+                         ("batch", 0, (32, 16)): 242.2}
 GB300_SMS = 152
 FP64_INST_PER_CLK_PER_SM = 2  # DFMA/DADD/DMUL issue rate of one SM (ncu peak_sustained)
 
@@ -708,7 +709,7 @@ def roofline_entry(args, r, peak, peak_src):
     instead: achieved FP64 instructions per second (where they have been
     counted) against the pipe's rate at the SM clock measured during the timed
     region."""
-    count = FP64_INST_PER_CELL_2D.get((args.workload, args.phase_model))
+    count = FP64_INST_PER_CELL_2D.get((args.workload, args.phase_model, tuple(r["cfg"]["tile"])))
     if args.workload == "batch" and args.batch_count < 64:
         count = None  # (fewer domains may run as 16 x 8 blocks)
     if r["prec"] == "p64" and r["kernel"] == "k_step2d" and count:

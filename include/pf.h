@@ -261,9 +261,11 @@ const char *pf_last_error(void);
  * domains with one persistent launch per step captured in a CUDA graph; the
  * kernel, tile shape and CTAs per SM are chosen by an autotuner (which times
  * the candidates on the live state) in the first step call of at least 256
- * steps, and cached per (dim, precision, size mix, domain count and the
- * features that decide which kernels can run it: walls, the Allen-Cahn
- * lattice, own contact angles, strip eligibility, unit relaxation rates); a
+ * steps, and cached per (dim, precision, cells to a power of two, domain
+ * count, number of free particles and the features that decide which kernels
+ * can run it: walls, the Allen-Cahn lattice, own contact angles, strip
+ * eligibility, unit relaxation rates; the segment rows of kernel 4 follow
+ * the sizes at hand); a
  * later batch of the same kind takes the cached configuration in its first
  * step call of any length.  Before that, steps run kernel 0.  Step calls
  * shorter than a 16-step chunk replay one-step graphs. */
@@ -312,8 +314,9 @@ int pf_batch_config(pf_batch *b, int *tile_x, int *tile_y, int *ctas_per_sm, int
  * paper).  tile_x x tile_y cells per tile; ctas_per_sm 0 = as many as fit,
  * else a cap.  kernel:
  *   0  one cell per thread (all policies, particles, walls, either
- *      order-parameter lattice; 2D tiles 32x8, 64x4, 32x16; 3D the tile
- *      of its policy);
+ *      order-parameter lattice; 2D tiles 32x8, 64x4, 32x16); 3D the step
+ *      and tile of its policy: in FP32 arithmetic without particles two
+ *      cells per thread, in two chunks of z, else one;
  *   1  2D, two vertically adjacent cells per thread in packed FP32
  *      arithmetic (P32 and PMIX, fixed solids, no walls, either lattice;
  *      tiles 32x16, 64x8, 32x32);

@@ -29,7 +29,7 @@ bool launch_step2d_p32(int tx, int ty, bool moving, int mode, int grid, cudaStre
 bool launch_step2d_mixh(int tx, int ty, bool moving, int mode, int grid, cudaStream_t s, const StepArgs &a, int *occ);
 bool launch_step2d_mixb(int tx, int ty, bool moving, int mode, int grid, cudaStream_t s, const StepArgs &a, int *occ);
 
-// 3D: one CTA marches through ZCHUNK3D planes in z
+// 3D: a tile marches through chunks of at most ZCHUNK3D planes in z
 constexpr int ZCHUNK3D = 32;
 bool launch_step3d(int prec, int tx, int ty, bool moving, int mode, int grid, cudaStream_t s,
                    const StepArgs &a);
@@ -45,8 +45,9 @@ void launch_init(int prec, const DomainDev &Dm, int *flags, const double *phi0, 
 int diag_blocks();
 // Launch with programmatic dependence on the kernel before it in the stream (the
 // kernel waits for it itself, see pdl_begin).  Per step in a graph, without and
-// with: 250 x 223 (FP32) 5.85 and 5.45 us, 16 particles in 512^2 39.4 and 35.7, the
-// strip step of 1024^2 between walls (with the queue's memset gone) 51.1 and 47.7.
+// with: 250 x 223 (FP32) 5.85 and 5.45 us, the strip step of 1024^2 between walls (with
+// the queue's memset gone) 51.1 and 47.7, 16 particles in 512^2 (step, repulsion and
+// update) 39.4 and about 36.
 template <class... K, class... A>
 inline void launch_pdl(void (*kern)(K...), int grid, int threads, int dyn, cudaStream_t s, const A &...args)
 {

@@ -20,10 +20,10 @@
 // that.  The frames of phi and phi0 are copied two planes ahead (cp.async); the
 // cell's own populations and lagged fields are loaded at the top of a plane
 // and used after its two barriers.
-// Measured per step, before and after: 256^3 with 16-bit storage 1399 -> 1060 us
-// (1140 instructions per cell), 131 x 100 x 90 in FP32 between walls 280 -> 125
-// us.  What bounds it now is issue: 2000 instructions per thread and plane at
-// 0.43 per clock and scheduler with 16 warps per SM, which registers cap.
+// Measured per step, before and after: 256^3 with 16-bit storage 1399 -> 1042 us
+// (1127 instructions per cell, 129 of them k_phi3d's), 131 x 100 x 90 in FP32 between
+// walls 280 -> 125 us.  What bounds it now is issue: 1996 instructions per thread and
+// plane at 0.44 per clock and scheduler with 16 warps per SM, which registers cap.
 // Constants pre-paired as float2 kernel parameters were slower (1115 us).
 #pragma once
 
